@@ -656,7 +656,7 @@ __global__ void groups_count_k(const int4 *cbox, const int4 *clink, const int *c
 // One warp per unit cell: writes its runs with their boxes from the scanned
 // offsets gofs (exclusive prefix of gcnt).
 __global__ void groups_write_k(const uint64_t *skey, const int4 *clink, const int *gofs, const int *gcnt_total,
-                               int G, int64_t cap, const DevState *st, int4 *groups) {
+                               int G, int64_t cap, const DevState *st, int4 *groups, int *garrive) {
     const int lane = threadIdx.x & 31;
     const int ncell = (int)min((int64_t)st->ncell, cap);
     const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
@@ -688,6 +688,7 @@ __global__ void groups_write_k(const uint64_t *skey, const int4 *clink, const in
                 const int g = g0 + r;
                 groups[2 * g] = make_int4(first, cnt, (int)qlo[0], (int)qlo[1]);
                 groups[2 * g + 1] = make_int4((int)qlo[2], (int)qhi[0], (int)qhi[1], (int)qhi[2]);
+                garrive[g] = 0;
             }
         }
     }
@@ -878,7 +879,7 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
     count_launch(c);
     if ((r = exclusive_scan(c, w.gcnt, c->cell_cap, &w.st->ncell, &w.st->ngroup, s)) != RV_OK) return r;
     groups_write_k<<<grid_for(c, c->cell_cap, 8), 256, 0, s>>>(skey, clink4, w.gcnt, &w.st->ngroup, G, c->cell_cap,
-                                                                w.st, w.groups);
+                                                                w.st, w.groups, w.garrive);
     count_launch(c);
     // multipoles
     moments_k<<<gb, 128, 0, s>>>(n, w.pos, w.cbox, w.clink, w.cparent, w.carrive, w.cmom, c->cell_cap, w.moff, M,

@@ -74,6 +74,10 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.gact = (uint8_t *)take(n + 1);
     t.scost = (float *)take(4 * n);
     t.gorder = (int *)take(4 * (n + 1));
+    t.gopart = (uint8_t *)take(n + 1);
+    t.garrive = (int *)take(4 * (n + 1));
+    // part sums: P(n) n slots, and P(n) n <= kPartItems group for every n with P(n) > 1
+    t.gpartial = (float4 *)take(16 * (size_t)std::min<int64_t>(kMaxParts * n, (int64_t)kPartItems * cfg.group));
     t.gbin = (int *)take(4 * (n + 1));
     t.obins = (int *)take(4 * 1024);
     t.block_count = (unsigned long long *)take(16);
@@ -511,7 +515,7 @@ rv_status rv_walk_stats(rv_ctx *c, int64_t out[3], void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long v[2];
     int hwm = 0;
-    cudaError_t e = cudaMemcpyAsync(v, &c->w.st->n_p2p, sizeof(v), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(v, &c->w.st->walk.n_p2p, sizeof(v), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hwm, &c->w.st->stack_hwm, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_check(c, e, "walk stats");

@@ -39,6 +39,35 @@ constexpr int kRedSlots = 1024;         // energy partial-sum blocks over all me
 constexpr int kMaxChain = 250;
 constexpr int kMaxPert = 5000;
 
+// Parts of a group's walk (walk.cu). In a small build the walk of every group is
+// split into P parts, each a work item of its own, so that few groups still
+// give every resident warp work: one warp takes 150 to 700 us for a group
+// whatever the system's size. P is the largest power of two that keeps the
+// items of n stars at or below kPartItems, six or seven for each of the 2432
+// resident warps; with more, the parts' repeated top of the traversal costs
+// more than the finer items balance, with fewer the last items run alone.
+// Walk in us on 65536 / 200001 stars (groups of 64, theta 0.5) with kPartItems
+// of 4096, 8192, 16384, 32768: 719, 614, 562, 643 / 1832, 1703, 1660, 1676;
+// unsplit 1286 / 1801.
+constexpr int kMaxParts = 16;
+constexpr int kPartItems = 16384;
+// Cells of more than 1 / kPartGrain of their member's stars are traversed by
+// every part (Part in walk.cu). Smaller subtrees balance better, larger ones
+// repeat less: 16000 / 65536 / 200001 stars took 169 / 593 / 1698 us at 32,
+// 150 / 562 / 1660 at 64, 158 / 581 / 1672 at 128, 172 / 589 / 1664 at 256.
+constexpr int kPartGrain = 64;
+__host__ __device__ __forceinline__ int parts_of(int64_t n, int group) {
+    const int64_t g = n / group + 1;
+    int P = 1;
+    while (P < kMaxParts && 2 * P * g <= kPartItems) P <<= 1;
+    return P;
+}
+// of a group with `count` stars: at most one part a star, so that the items are at most n
+__host__ __device__ __forceinline__ int parts_of_group(int P, int count) {
+    while (P > count) P >>= 1;
+    return P;
+}
+
 // Error codes latched by kernels (first one wins).
 enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kErrPairs = 4, kErrTimeout = 5 };
 
@@ -46,13 +75,15 @@ enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kE
 struct DevState {
     int ncell;        // cells of the last build
     int ngroup;       // walk groups of the last build
-    int next_group;   // walk work counter
     int err;          // latched DevErr
     int n_pert;       // perturbers selected by the last selection
     int stack_hwm;    // deepest walk stack seen
     int cost_n;       // stars whose walk costs scost holds (0: none)
-    int pad;
-    unsigned long long n_p2p, n_m2p;  // interaction counts of the last walk
+    struct {          // zeroed before every walk
+        int next_item;    // walk work counter
+        int nitem;        // work items in the queue order (0 until the order is made)
+        unsigned long long n_p2p, n_m2p;  // interaction counts of the last walk
+    } walk;
     double bounds[5];                 // min x, y, z, L, 2^21 / L
     double absorb[4];                 // chain absorption: centre of mass x, y, z and the squared chain radius
     int lvoff[kLevels + 1];           // first cell of each level, then ncell
@@ -77,7 +108,10 @@ struct Workspace {
     int4 *groups;         // 2 int4 per group: (first, count, lo x, lo y), (lo z, hi x, hi y, hi z)
     uint8_t *gact;        // block time steps: groups holding an active star
     float *scost;         // per caller star: list cost of its group in the last walk (scheduling only)
-    int *gorder;          // the walk's queue order of the groups
+    int *gorder;          // the walk's queue order of the work items: each one's group
+    uint8_t *gopart;      // ... and its part of the group's walk
+    int *garrive;         // parts of each group's walk that are done
+    float4 *gpartial;     // part sums of the stars of groups walked in several parts [part][sorted star]
     int *gbin;            // each group's cost bin (queue order scratch)
     int *obins;           // bin counts, then next free slots (queue order scratch, 1024)
     unsigned long long *block_count;  // block time steps: active star updates so far
@@ -128,6 +162,7 @@ struct rv_ctx {
     int n_walk_events;
     int cap_walk_events;
     cudaEvent_t *walk_events;               // [2 cap_walk_events]
+    int walk_blocks[16];                    // resident walk blocks of each kernel variant (0: not asked yet)
     // captured kick-drift-kick step (rv_kdk_step_graph)
     cudaGraphExec_t graph;
     long long graph_launches;

@@ -1,11 +1,11 @@
 // walk.cu -- Barnes-Hut tree walk and interaction evaluation (FP32).
 //
-// One warp walks the tree for one group of up to 64 consecutive stars. Cells
-// are tested up to 64 a pass, two per lane, under the box-box opening test;
-// accepted cells are staged in shared memory as multipole records, opened
-// leaves stage their stars, opened internal cells push their child range on
-// a per-warp stack. Whenever a staged list holds a full tile, the warp
-// evaluates it: a lane holds two stars of the group (a target pair), each of
+// One warp walks the tree for one group of up to 64 consecutive stars, or, in
+// small builds, for one part of a group's walk (Part). Cells are tested up to 64
+// a pass, two per lane, under the box-box opening test; accepted cells are
+// staged in shared memory as multipole records, opened leaves stage their
+// stars, opened internal cells push their child range on a per-warp stack.
+// Whenever a staged list holds a full tile, the warp evaluates it: a lane holds two stars of the group (a target pair), each of
 // the p = ceil(s / 2) pairs is served by k = floor(32 / p) lanes, lane t + i p
 // taking list pairs i, i + k, ... with broadcast shared-memory reads and
 // evaluating every loaded source pair on both its stars; tile sums are added
@@ -16,11 +16,9 @@
 //
 // Staged lists hold list entries in pairs, each field of the two entries
 // side by side, so that one lane evaluates two interactions with the packed
-// two-wide FP32 instructions (add/mul/fma .f32x2): the walk is bound by
-// instruction issue, and a packed instruction does two lanes' worth of FP32
-// work in one issue slot. Each interaction is still computed element by
-// element in FP32 round-to-nearest; only the order of the running sums
-// differs from one entry per instruction.
+// two-wide FP32 instructions (add/mul/fma .f32x2). Each interaction is still
+// computed element by element in FP32 round-to-nearest; only the order of the
+// running sums differs from one entry per instruction.
 //
 // Interactions (G = 1, Sect. 3 Plummer softening; multipoles about the cell's
 // centre of mass, Sect. 1):
@@ -34,22 +32,30 @@
 
 #include "rv_internal.cuh"
 
+// What bounds it: instruction dispatch. A packed FP32 instruction takes two
+// dispatch cycles of its scheduler and every other instruction at least one
+// (the evaluation loop alone, any number of warps from 8 an SM up, reaches 0.82
+// of the FMA peak for cells and 0.71 for stars: 132 + ~27 and 52 + ~19 cycles an
+// iteration), so a pass that tests, stages and evaluates is worth what its
+// instructions add up to; on 2^20 stars at theta 0.5 the packed instructions
+// are 75 % of the walk's dispatch cycles.
+//
 // Unrolling of the evaluation loops (list pairs in flight per lane, each on
-// two targets; measured on GB300: star pairs 1, cell pairs 3) and the
-// register budget of the walk kernel. The kernel runs one warp per block, so
-// the register budget alone sets the resident warps: 104 registers a thread
-// (the running sums live in shared memory) give 18-19 warps per SM, against
-// 16 at 128 registers; 96 registers spill, 112 and 128 were slower
-// (2^24 stars at theta 0.8 and tile 96: 80.9 ms at 104 registers, 84.8 at
-// 112, 84.8 at 128, 88.6 at 96).
+// two targets; measured on GB300: star pairs 1, cell pairs 4, which also divides
+// every tile) and the register budget of the walk kernel. The kernel runs one
+// warp per block; 112 registers a thread (the running sums and what a work item
+// needs at its end live in shared memory) give 16 warps per SM, as 104 and 128
+// do, and nothing spills. Walk of 2^20 stars at theta 0.5 / 2^22 at 0.8, tile 96:
+// 8.50 / 18.3 ms at 112, 8.69 / 18.8 at 104, 9.07 / 19.7 at 120, 9.2 / 19.9 at
+// 128; cell pairs 2, 3, 4 at 112: 8.86, 8.52, 8.50 ms.
 #ifndef RV_P2P_UNROLL
 #define RV_P2P_UNROLL 1
 #endif
 #ifndef RV_M2P_UNROLL
-#define RV_M2P_UNROLL 3
+#define RV_M2P_UNROLL 4
 #endif
 #ifndef RV_WALK_MAXNREG
-#define RV_WALK_MAXNREG 104
+#define RV_WALK_MAXNREG 112
 #endif
 #ifdef RV_WALK_MIN_BLOCKS
 #define RV_WALK_BOUNDS __launch_bounds__(kWalkWarps * 32, RV_WALK_MIN_BLOCKS)
@@ -102,28 +108,33 @@ struct WalkArgs {
     const float *arx, *ary, *arz;
     // optional group mask (block time steps): only groups with gact[g] != 0 are walked
     const uint8_t *gact;
-    // queue order of the groups (null: build order), and the per-star list cost
-    // written for the next walk's order
+    // queue order of the work items (null: build order, `parts` items a group),
+    // and the per-star list cost written for the next walk's order
     const int *order;
+    const uint8_t *opart;
     float *scost;
+    // parts of the groups' walks (Part)
+    int parts, n_leaf;
+    float4 *partial;   // [part][sorted star]
+    int *garrive;
     // spline softening of the stars (h = 2.8 eps)
     Spline spl;
     // the walk stack's entries beyond kStackSm: kStackSpill per warp of the launch
     int *gstack;
 };
 
-// Per-warp shared memory: stack | lane_cell[32] | cell staging | star staging |
-// running sums. Cell staging: (tile + 32) / 2 pairs of multipole records, 5
+// Per-warp shared memory: stack | lf_delta[64] | cell staging | star staging |
+// running sums. Cell staging: (tile + 64) / 2 pairs of multipole records, 5
 // float4 per pair holding (M, cx), (cy, cz), (-Qxx, -Qyy), (-Qzz, -Qxy),
 // (-Qxz, -Qyz) of both entries side by side (cx.. = centre of mass relative
-// to the group centre). Star staging: (tile + 32) / 2 pairs, 2 float4 per
+// to the group centre). Star staging: (tile + 64) / 2 pairs, 2 float4 per
 // pair: (x, y), (z, m). Running sums: 16 floats per lane (AccSm).
 constexpr int kCellPairF4 = 5, kStarPairF4 = 2;
 constexpr int kAccWords = 16 * 32;
 constexpr int kP2PUnroll = RV_P2P_UNROLL, kM2PUnroll = RV_M2P_UNROLL;
 __host__ __device__ inline size_t warp_staging_bytes(int tile) {
-    return (size_t)kStackSm * 4 + 192 * 4 + (size_t)(tile + 64) / 2 * 16 * kCellPairF4 +
-           (size_t)(tile + 32) / 2 * 16 * kStarPairF4;
+    return (size_t)kStackSm * 4 + 64 * 4 + (size_t)(tile + 64) / 2 * 16 * kCellPairF4 +
+           (size_t)(tile + 64) / 2 * 16 * kStarPairF4;
 }
 __host__ __device__ inline size_t warp_smem_bytes(int tile) { return warp_staging_bytes(tile) + 4 * kAccWords; }
 
@@ -436,11 +447,42 @@ __device__ __forceinline__ void pad_stars(float4 *p2p, int cnt) {
     }
 }
 
-__device__ __forceinline__ int gap1(int blo, int bhi, int clo, int chi) {
-    return (clo >= bhi) ? clo - bhi : ((blo >= chi) ? blo - chi : 0);
+__device__ __forceinline__ unsigned gap1(int blo, int bhi, int clo, int chi) {
+    return (unsigned)max(max(clo - bhi, blo - chi), 0);
 }
 
-// Walks the tree for one group; returns false if a bound was violated.
+// The `mv` (<= 32) pairs from pair `from` on to the front of a staged list, field
+// by field. Source and destination overlap when from < mv (tiles below 64
+// entries): then every read of a field before its writes.
+template <int F4>
+__device__ __forceinline__ void move_front(float4 *list, int from, int mv) {
+    const int lane = threadIdx.x & 31;
+    const float4 *src = list + F4 * (from + lane);
+    float4 *dst = list + F4 * lane;
+#pragma unroll
+    for (int f = 0; f < F4; f++) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < mv) v = src[f];
+        if (from < 32) __syncwarp();
+        if (lane < mv) dst[f] = v;
+        if (from < 32) __syncwarp();
+    }
+    __syncwarp();
+}
+
+// A work item's share of its group's walk: part q of P (P a power of two, pm =
+// P - 1). Cells of more than `big` stars are traversed by every part; a cell at
+// or below that size reached from a bigger one belongs, with everything under
+// it, to part (its first star within its member) mod P, and so does every bigger
+// cell that is accepted or is a leaf. The split depends on P and the member's
+// tree alone, so a group's sums do not depend on which warps walk its parts, on
+// the order they finish in or on a group mask. own = (part + member's first
+// star) mod P; P = 1: pm = 0, own = 0, big = -1.
+struct Part {
+    int own, pm, big;
+};
+
+// Walks one part of the tree for one group; returns false if a bound was violated.
 // Positions in the walk are relative to g, the geometric centre of the
 // group's box: targets and staged sources are shifted once, cell centres of
 // mass are (cell centre - g) + (centre of mass - cell centre). Differences of
@@ -450,23 +492,24 @@ template <bool SOFT, bool QUAD, bool REC, bool REL, bool SPL>
 __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, const unsigned long long *thr,
                                            const unsigned long long *thr_rec, int gid, char *wsm, const int blo[3],
                                            const int bhi[3], const float g[3], const Tgt &tg, f2 eps2, const AccSm &acc,
-                                           unsigned long long &np2p, unsigned long long &nm2p, float K) {
+                                           const Part &part, unsigned &np2p, unsigned &nm2p, float K) {
     const int lane = threadIdx.x & 31;
     const int T = A.tile;
     // the range stack: entries below kStackSm in shared memory, the deeper ones
-    // (rare: a pass pushes at most 32, and the walk is depth-first) in this
-    // warp's spill area in global memory; __syncwarp orders both for the warp
+    // (rare: a pass pushes at most 64, and the walk is depth-first) in this
+    // warp's spill area in global memory; __syncwarp orders both for the warp.
+    // An entry is a child range (first << 4 | owned << 3 | count - 1); `owned`:
+    // the part owns everything under it.
     int *stack = reinterpret_cast<int *>(wsm);
-    int *spill = A.gstack + (size_t)(blockIdx.x * kWalkWarps + (threadIdx.x >> 5)) * kStackSpill;
-    auto st_get = [&](int i) -> int { return i < kStackSm ? stack[i] : spill[i - kStackSm]; };
-    int *lane_cell = stack + kStackSm;                             // a pass's 64 cells
-    int *lf_first = lane_cell + 64, *lf_start = lane_cell + 128;   // a pass's opened leaves
-    float4 *m2p = reinterpret_cast<float4 *>(lane_cell + 192);
+    const unsigned spill0 = (blockIdx.x * kWalkWarps + (threadIdx.x >> 5)) * kStackSpill - kStackSm;
+    static_assert((size_t)kStackSpillWarps * kStackSpill < 1u << 31, "32-bit spill offsets");
+    int *lf_delta = stack + kStackSm;   // a pass's opened leaves: first star minus its place among the pass's stars
+    float4 *m2p = reinterpret_cast<float4 *>(lf_delta + 64);
     float4 *p2p = m2p + kCellPairF4 * ((T + 64) / 2);
-    const unsigned lt = lanemask_lt();
+    const unsigned lt = lanemask_lt(), le = (lt << 1) | 1u;
     const int ncell = G.ncell;
 
-    if (lane == 0) stack[0] = (G.root << 4) | 1;  // the member's root: a range of one cell
+    if (lane == 0) stack[0] = G.root << 4;  // the member's root: a range of one cell
     int top = 1, nm = 0, np = 0, hwm = 1;
     bool ok = true;
     // every pass tests at least one new cell, so a walk ends within ncell passes
@@ -475,36 +518,34 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
     // a cell's records, opening test and link check (one of a pass's two slots per lane)
     struct Slot {
         int c;
-        bool accept, leaf, open, band;
+        bool owned, accept, leaf, open, band;
         int4 lk, b;
-        float4 r0, q1, q2;
+        float4 r0, q1;
+        float2 q2;
     };
     auto load_slot = [&](Slot &x) {
-        x.accept = x.leaf = x.open = x.band = false;
-        x.lk = make_int4(0, 0, 0, 0);
-        x.b = make_int4(0, 0, 0, 0);
-        x.r0 = make_float4(0.f, 0.f, 0.f, 0.f);
-        x.q1 = x.r0;
-        x.q2 = x.r0;
-        if (x.c >= 0) {
-            // every record of the cell at once: one L2 round trip per pass
-            x.b = __ldg(&A.cbox[x.c]);
-            x.lk = __ldg(&A.clink[x.c]);
-            x.r0 = __ldg(&A.cmom[3 * x.c + 0]);
-            if (QUAD) {
-                x.q1 = __ldg(&A.cmom[3 * x.c + 1]);
-                x.q2 = __ldg(&A.cmom[3 * x.c + 2]);
-            }
+        // every record of the cell at once: one L2 round trip per pass. A slot
+        // without a cell (c < 0), or with a bad index, reads the first or last cell's.
+        const int c = min(max(x.c, 0), ncell - 1);
+        x.b = __ldg(&A.cbox[c]);
+        x.lk = __ldg(&A.clink[c]);
+        x.r0 = __ldg(&A.cmom[3 * c + 0]);
+        if (QUAD) {
+            x.q1 = __ldg(&A.cmom[3 * c + 1]);
+            x.q2 = __ldg(reinterpret_cast<const float2 *>(&A.cmom[3 * c + 2]));
         }
     };
     auto test_slot = [&](Slot &x) -> bool {   // returns "bad link"
+        x.accept = x.leaf = x.open = x.band = false;
+        bool bad = x.c >= ncell;
         if (x.c >= 0) {
             const int4 b = x.b;
             const int side = 1 << (kMaxLevel - b.w);
-            const long long gx = gap1(blo[0], bhi[0], b.x, b.x + side);
-            const long long gy = gap1(blo[1], bhi[1], b.y, b.y + side);
-            const long long gz = gap1(blo[2], bhi[2], b.z, b.z + side);
-            const unsigned long long d2 = (unsigned long long)(gx * gx + gy * gy + gz * gz);
+            const unsigned gx = gap1(blo[0], bhi[0], b.x, b.x + side);
+            const unsigned gy = gap1(blo[1], bhi[1], b.y, b.y + side);
+            const unsigned gz = gap1(blo[2], bhi[2], b.z, b.z + side);
+            const unsigned long long d2 = (unsigned long long)gx * gx + (unsigned long long)gy * gy +
+                                          (unsigned long long)gz * gz;
             if (REL && K >= 0.f) {
                 // relative criterion: the group's box outside the cell's box grown by
                 // side/10 per side (integers x 10), and M s^2 <= (K d^2) d^2 in FP32
@@ -519,15 +560,23 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
             } else {
                 x.accept = d2 >= thr[b.w];
             }
-            if (REC) x.band = x.accept && d2 < thr_rec[b.w];
-            if (!x.accept) {
-                x.leaf = (x.lk.x == x.lk.y);
-                x.open = !x.leaf;
+            const bool mine = x.owned || ((x.lk.z & part.pm) == part.own);
+            if (x.accept) {
+                if (REC) x.band = mine && d2 < thr_rec[b.w];
+                x.accept = mine;
+            } else if (x.lk.x == x.lk.y) {
+                x.leaf = mine;
+                // links must stay inside the tree (a violated bound ends the walk with an error)
+                bad |= (unsigned)x.lk.w > (unsigned)A.n || (unsigned)x.lk.z > (unsigned)x.lk.w;
+            } else {
+                // (a range's end is checked cell by cell, when they are popped)
+                bad |= x.lk.x <= x.c || (unsigned)(x.lk.y - x.lk.x) > 8u;
+                const bool shared = !x.owned && x.lk.w - x.lk.z > part.big;
+                x.open = shared || mine;
+                x.owned = !shared;   // of the children
             }
         }
-        // links must stay inside the tree (a violated bound ends the walk with an error)
-        return (x.open && (x.lk.x <= x.c || x.lk.y > ncell || x.lk.y - x.lk.x > 8)) ||
-               (x.leaf && (x.lk.z < 0 || x.lk.w > A.n || x.lk.z > x.lk.w));
+        return bad;
     };
     auto stage_cell = [&](const Slot &x, int p) {
         float c0[3];
@@ -545,59 +594,65 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
             *staged(m2p, kCellPairF4, p, 9) = -x.q2.y;
         }
     };
-    auto push = [&](int p, const int4 lk) {
-        if (p < kStackSm) stack[p] = (lk.x << 4) | (lk.y - lk.x);
-        else if (p < kStackCap) spill[p - kStackSm] = (lk.x << 4) | (lk.y - lk.x);
+    auto push = [&](int p, const Slot &x) {
+        const int e = (x.lk.x << 4) | (x.owned ? 8 : 0) | (x.lk.y - x.lk.x - 1);
+        if (p < kStackSm) stack[p] = e;
+        else if (p < kStackCap) A.gstack[spill0 + p] = e;
     };
     while (top > 0) {
         if (--guard < 0) { ok = false; break; }
         // pop whole child ranges from the top while they fit in the pass's 64
-        // slots (slot s: lane s % 32, its first or second cell)
+        // slots (slot s: lane s % 32, its first or second cell). Lane i holds
+        // ranges i and i + 32 from the top; both prefix sums of their lengths run
+        // in one register (16 bits each), and a slot finds its range from the
+        // 64-bit mask of the ranges' first slots: its rank is the number of ranges
+        // starting at or before it (a warp OR and a population count, instead of
+        // writing the cells to shared memory and reading them back).
         const int avail = min(top, 64);
-        const int e0 = (lane < avail) ? st_get(top - 1 - lane) : 0;
-        const int e1 = (lane + 32 < avail) ? st_get(top - 33 - lane) : 0;
-        const int n0 = e0 & 15, n1 = e1 & 15;
-        int in0 = n0, in1 = n1;
+        const int i0 = top - 1 - lane, i1 = top - 33 - lane;
+        int e0 = stack[min(max(i0, 0), kStackSm - 1)], e1 = stack[min(max(i1, 0), kStackSm - 1)];
+        if (top > kStackSm) {
+            if (i0 >= kStackSm) e0 = A.gstack[spill0 + i0];
+            if (i1 >= kStackSm) e1 = A.gstack[spill0 + i1];
+        }
+        const int n0 = (lane < avail) ? (e0 & 7) + 1 : 0, n1 = (lane + 32 < avail) ? (e1 & 7) + 1 : 0;
+        unsigned in = (unsigned)n0 | ((unsigned)n1 << 16);
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y0 = __shfl_up_sync(0xffffffffu, in0, o);
-            const int y1 = __shfl_up_sync(0xffffffffu, in1, o);
-            if (lane >= o) {
-                in0 += y0;
-                in1 += y1;
-            }
+            const unsigned y = __shfl_up_sync(0xffffffffu, in, o);
+            if (lane >= o) in += y;
         }
-        in1 += __shfl_sync(0xffffffffu, in0, 31);
-        const unsigned fit0 = __ballot_sync(0xffffffffu, lane < avail && in0 <= 64);
-        const unsigned fit1 = __ballot_sync(0xffffffffu, lane + 32 < avail && in1 <= 64);
-        const int kk = __popc(fit0) + __popc(fit1);
-        const int tA = __shfl_sync(0xffffffffu, in0, min(kk, 32) - 1);
-        const int tB = __shfl_sync(0xffffffffu, in1, max(kk - 33, 0));
-        const int total = kk <= 32 ? tA : tB;
-        __syncwarp();
-        if (lane < kk) {
-            const int b0 = in0 - n0, c0 = e0 >> 4;
-            for (int t = 0; t < n0; t++) lane_cell[b0 + t] = c0 + t;
-        }
-        if (lane + 32 < kk) {
-            const int b1 = in1 - n1, c1 = e1 >> 4;
-            for (int t = 0; t < n1; t++) lane_cell[b1 + t] = c1 + t;
-        }
-        top -= kk;
-        __syncwarp();
+        const int in0 = in & 0xffff, in1 = (in >> 16) + (__shfl_sync(0xffffffffu, in, 31) & 0xffff);
+        const bool fit0 = n0 > 0 && in0 <= 64, fit1 = n1 > 0 && in1 <= 64;
+        const int s0 = in0 - n0, s1 = in1 - n1;
+        const unsigned mlo = __reduce_or_sync(0xffffffffu, (fit0 && s0 < 32 ? 1u << (s0 & 31) : 0u) |
+                                                               (fit1 && s1 < 32 ? 1u << (s1 & 31) : 0u));
+        const unsigned mhi = __reduce_or_sync(0xffffffffu, (fit0 && s0 >= 32 ? 1u << (s0 & 31) : 0u) |
+                                                               (fit1 && s1 >= 32 ? 1u << (s1 & 31) : 0u));
+        const int total = __reduce_max_sync(0xffffffffu, max(fit0 ? in0 : 0, fit1 ? in1 : 0));
+        const int klo = __popc(mlo);
+        top -= klo + __popc(mhi);
         Slot xa, xb;
-        xa.c = (lane < total) ? lane_cell[lane] : -1;
-        xb.c = (lane + 32 < total) ? lane_cell[lane + 32] : -1;
-        __syncwarp();
-        if (__any_sync(0xffffffffu, xa.c >= ncell || xb.c >= ncell)) { ok = false; break; }
+        {
+            const unsigned ma = mlo & le, mb = mhi & le;
+            const int ra = __popc(ma) - 1, rb = klo + __popc(mb) - 1;   // ranks of the slots' ranges (slot 0 starts one)
+            const int sa = 31 - __clz(ma), sb = mb ? 63 - __clz(mb) : 31 - __clz(mlo);
+            const int ea = __shfl_sync(0xffffffffu, e0, ra);
+            const int eb0 = __shfl_sync(0xffffffffu, e0, rb & 31), eb1 = __shfl_sync(0xffffffffu, e1, rb & 31);
+            const int eb = rb < 32 ? eb0 : eb1;
+            xa.c = (lane < total) ? (ea >> 4) + (lane - sa) : -1;
+            xb.c = (lane + 32 < total) ? (eb >> 4) + (lane + 32 - sb) : -1;
+            xa.owned = (ea & 8) != 0;
+            xb.owned = (eb & 8) != 0;
+        }
         load_slot(xa);
         load_slot(xb);
         const bool bad_a = test_slot(xa), bad_b = test_slot(xb);
         if (__any_sync(0xffffffffu, bad_a || bad_b)) { ok = false; break; }
         // opened internal cells: push their child ranges (slot order)
         const unsigned oma = __ballot_sync(0xffffffffu, xa.open), omb = __ballot_sync(0xffffffffu, xb.open);
-        if (xa.open) push(top + __popc(oma & lt), xa.lk);
-        if (xb.open) push(top + __popc(oma) + __popc(omb & lt), xb.lk);
+        if (xa.open) push(top + __popc(oma & lt), xa);
+        if (xb.open) push(top + __popc(oma) + __popc(omb & lt), xb);
         top += __popc(oma) + __popc(omb);
         hwm = max(hwm, top);
         if (top > kStackCap) { ok = false; break; }
@@ -627,66 +682,75 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
         }
         // opened leaves: stage their stars relative to g, leaves in slot order
         // and stars in order within each (the order the tiles take them), 32
-        // stars a round whichever leaves they come from, so that the loads of
-        // a pass's leaves overlap instead of following one another
+        // stars a round whichever leaves they come from, two rounds' loads in
+        // flight; a star finds its leaf as a slot finds its range
         const unsigned lma = __ballot_sync(0xffffffffu, xa.leaf), lmb = __ballot_sync(0xffffffffu, xb.leaf);
         if (lma | lmb) {
             const int ca = xa.leaf ? xa.lk.w - xa.lk.z : 0, cb = xb.leaf ? xb.lk.w - xb.lk.z : 0;
-            int ia = ca, ib = cb;
+            int ia, ib;
+            if (__any_sync(0xffffffffu, max(ca, cb) > 2047)) {   // overfull leaves of the finest level
+                ia = ca;
+                ib = cb;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int ya = __shfl_up_sync(0xffffffffu, ia, o);
-                const int yb = __shfl_up_sync(0xffffffffu, ib, o);
-                if (lane >= o) {
-                    ia += ya;
-                    ib += yb;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int ya = __shfl_up_sync(0xffffffffu, ia, o);
+                    const int yb = __shfl_up_sync(0xffffffffu, ib, o);
+                    if (lane >= o) {
+                        ia += ya;
+                        ib += yb;
+                    }
                 }
+            } else {   // both sums below 2^16
+                unsigned iab = (unsigned)ca | ((unsigned)cb << 16);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, iab, o);
+                    if (lane >= o) iab += y;
+                }
+                ia = (int)(iab & 0xffff);
+                ib = (int)(iab >> 16);
             }
             ib += __shfl_sync(0xffffffffu, ia, 31);
             const int total_stars = __shfl_sync(0xffffffffu, ib, 31);
-            const int nla = __popc(lma), nl = nla + __popc(lmb);
-            if (xa.leaf) {
-                const int k = __popc(lma & lt);
-                lf_first[k] = xa.lk.z;
-                lf_start[k] = ia - ca;
-            }
-            if (xb.leaf) {
-                const int k = nla + __popc(lmb & lt);
-                lf_first[k] = xb.lk.z;
-                lf_start[k] = ib - cb;
-            }
+            const int sa = xa.leaf ? ia - ca : -1, sb = xb.leaf ? ib - cb : -1;   // -1: no window holds it
+            if (xa.leaf) lf_delta[__popc(lma & lt)] = xa.lk.z - sa;
+            if (xb.leaf) lf_delta[__popc(lma) + __popc(lmb & lt)] = xb.lk.z - sb;
             __syncwarp();
-            for (int base = 0; base < total_stars; base += 32) {
-                const int idx = base + lane, cc = min(32, total_stars - base);
-                if (lane < cc) {
-                    // the leaf holding star idx of the pass: the last one starting at or before idx
-                    int lo = 0, hi = nl - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (lf_start[mid] <= idx) lo = mid; else hi = mid - 1;
-                    }
-                    const float4 s = __ldg(&A.pos[lf_first[lo] + (idx - lf_start[lo])]);
-                    const int e = np + lane;
-                    *staged(p2p, kStarPairF4, e, 0) = s.x - g[0];
-                    *staged(p2p, kStarPairF4, e, 1) = s.y - g[1];
-                    *staged(p2p, kStarPairF4, e, 2) = s.z - g[2];
-                    *staged(p2p, kStarPairF4, e, 3) = s.w;
+            int before = -1;   // leaves that started before the window, minus one
+            for (int base = 0; base < total_stars; base += 64) {
+                float4 st2[2];
+                int cc[2];
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int w0 = base + 32 * h, idx = w0 + lane;
+                    cc[h] = min(32, total_stars - w0);   // <= 0: no second round
+                    const unsigned m = __reduce_or_sync(
+                        0xffffffffu, ((unsigned)(sa - w0) < 32u && sa >= 0 ? 1u << (sa - w0) : 0u) |
+                                         ((unsigned)(sb - w0) < 32u && sb >= 0 ? 1u << (sb - w0) : 0u));
+                    if (lane < cc[h]) st2[h] = __ldg(&A.pos[lf_delta[before + __popc(m & le)] + idx]);
+                    before += __popc(m);
                 }
-                np += cc;
-                np2p += cc;
-                if (np >= T) {
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    if (lane < cc[h]) {
+                        const int e = np + lane;
+                        *staged(p2p, kStarPairF4, e, 0) = st2[h].x - g[0];
+                        *staged(p2p, kStarPairF4, e, 1) = st2[h].y - g[1];
+                        *staged(p2p, kStarPairF4, e, 2) = st2[h].z - g[2];
+                        *staged(p2p, kStarPairF4, e, 3) = st2[h].w;
+                    }
+                    np += max(cc[h], 0);
+                }
+                // np < T before the two rounds, so at most T + 63 entries are ever staged
+                while (np >= T) {
                     __syncwarp();
                     eval_p2p<SOFT, SPL>(p2p, T / 2, tg, eps2, A.spl, acc);
                     __syncwarp();
-                    // T is even: the leftover entries move pair by pair
-                    if (lane < (np - T + 1) / 2) {
-                        p2p[kStarPairF4 * lane] = p2p[kStarPairF4 * (T / 2 + lane)];
-                        p2p[kStarPairF4 * lane + 1] = p2p[kStarPairF4 * (T / 2 + lane) + 1];
-                    }
+                    move_front<kStarPairF4>(p2p, T / 2, (np - T + 1) / 2);
                     np -= T;
-                    __syncwarp();
                 }
             }
+            np2p += total_stars;
         }
         // a pass adds up to 64 cells: flush while a full tile is staged (nm < T
         // before every pass, so at most T + 63 entries are ever staged)
@@ -694,15 +758,7 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
             __syncwarp();
             eval_m2p<QUAD, SPL>(m2p, T / 2, tg, eps2, A.spl, acc);
             __syncwarp();
-            // the leftover (up to 32 pairs) to the front; read all before writing any,
-            // as source and destination overlap when T < 64
-            const int mv = (nm - T + 1) / 2;
-            for (int f = 0; f < kCellPairF4; f++) {   // field by field: every read of a field before its writes
-                const float4 v = lane < mv ? m2p[kCellPairF4 * (T / 2 + lane) + f] : make_float4(0.f, 0.f, 0.f, 0.f);
-                __syncwarp();
-                if (lane < mv) m2p[kCellPairF4 * lane + f] = v;
-                __syncwarp();
-            }
+            move_front<kCellPairF4>(m2p, T / 2, (nm - T + 1) / 2);
             nm -= T;
         }
         __syncwarp();
@@ -718,6 +774,13 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
     __syncwarp();
     if (lane == 0) atomicMax(&A.st->stack_hwm, hwm);
     return ok;
+}
+
+// Zeroes the warp's running sums.
+__device__ __forceinline__ void clear_acc(float *accw) {
+#pragma unroll
+    for (int k = 0; k < 16; k++) accw[32 * k + (threadIdx.x & 31)] = 0.f;
+    __syncwarp();
 }
 
 // Lane l serves target pair t = l % p (stars 2t and 2t + 1) with share
@@ -787,9 +850,47 @@ __device__ __forceinline__ void extra_terms(const WalkArgs &A, float xi, float y
     nadd(acc.ax, acc.cx, tx); nadd(acc.ay, acc.cy, ty); nadd(acc.az, acc.cz, tz); nadd(acc.ph, acc.cp, tp);
 }
 
-// Work items 0 .. n_extra-1 are the extra particles (one-star groups whose box
-// is their own grid cell [q, q+1)^3, q = floor((x - min) 2^21 / L) limited
-// to +-2^23); the tree's groups follow.
+// A part of a walk is done: true in the warp that finishes the last of the P
+// parts (whose sums every part has then written), which also resets the counter.
+__device__ __forceinline__ bool last_part(int *arrive, int P) {
+    int last = 0;
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        __threadfence();   // this part's sums before its arrival
+        last = atomicAdd(arrive, 1) == P - 1;
+        if (last) *arrive = 0;
+        __threadfence();
+    }
+    return __shfl_sync(0xffffffffu, last, 0) != 0;
+}
+
+__device__ __forceinline__ float4 part_sum(const Acc &t) {
+    return make_float4(t.ax + t.cx, t.ay + t.cy, t.az + t.cz, t.ph + t.cp);
+}
+
+// The parts' sums added in part order (p: the first part's slot, the next ones `stride` apart).
+__device__ __forceinline__ Acc add_parts(const float4 *p, int64_t stride, int P) {
+    Acc t = {};
+    for (int q = 0; q < P; q++) {
+        const float4 v = __ldcg(p + q * stride);
+        nadd(t.ax, t.cx, v.x); nadd(t.ay, t.cy, v.y); nadd(t.az, t.cz, v.z); nadd(t.ph, t.cp, v.w);
+    }
+    return t;
+}
+
+__device__ __forceinline__ Part part_of(int q, int P, int64_t m0, int64_t n_member, int n_leaf) {
+    const int grain = (int)(n_member / kPartGrain);
+    return Part{(int)((q + m0) & (P - 1)), P - 1, P > 1 ? max(n_leaf, grain) : -1};
+}
+
+// A work item of a group, as the warp keeps it in shared memory while it walks.
+struct Item {
+    int group, first, count, member, q, P;
+};
+
+// Work items: the extra particles (one-star groups whose box is their own grid
+// cell [q, q+1)^3, q = floor((x - min) 2^21 / L) limited to +-2^23; never split:
+// FP64 quantities are made from their forces), then the tree's groups in their parts.
 template <bool SOFT, bool QUAD, bool REC, bool REL, bool SPL>
 __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
     extern __shared__ __align__(16) char smem[];
@@ -798,23 +899,20 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
     // of different levels, which a constant-bank read would serialise
     __shared__ unsigned long long mac_thr[kLevels];
     __shared__ unsigned long long rec_thr[REC ? kLevels : 1];
+    __shared__ Item item[kWalkWarps];
     if (threadIdx.x < kLevels) mac_thr[threadIdx.x] = A.mac.thr[threadIdx.x];
     if (REC && threadIdx.x < kLevels) rec_thr[threadIdx.x] = A.rec.thr[threadIdx.x];
     __syncthreads();
     char *wsm = smem + wib * warp_smem_bytes(A.tile);
-    const int nitem = A.n_extra + A.st->ngroup;
-    unsigned long long np2p = 0, nm2p = 0;
+    const int nitem = A.n_extra + (A.order ? A.st->walk.nitem : A.st->ngroup * A.parts);
     while (true) {
         int gi = 0;
-        if (lane == 0) gi = atomicAdd(&A.st->next_group, 1);
+        if (lane == 0) gi = atomicAdd(&A.st->walk.next_item, 1);
         gi = __shfl_sync(0xffffffffu, gi, 0);
         if (gi >= nitem) break;
         float *accw = reinterpret_cast<float *>(wsm + warp_staging_bytes(A.tile));
         const AccSm acc{accw + lane};
-#pragma unroll
-        for (int k = 0; k < 16; k++) accw[32 * k + lane] = 0.f;
-        __syncwarp();
-        unsigned long long a2 = 0, a3 = 0;
+        unsigned a2 = 0, a3 = 0;   // list entries of the group: stars, cells
         if (gi < A.n_extra) {
             // ---- a particle outside the tree: all 32 lanes share its interaction list
             // (both target slots hold it; the second slot's sums are not used)
@@ -841,10 +939,11 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
             tg.nz[0] = tg.nz[1] = f2_pack(g[2] - zi, g[2] - zi);
             tg.j0 = lane;
             tg.k = 32;
+            clear_acc(accw);
             bool ok = true;
             if (G.ncell > 0 && G.root >= 0)
                 ok = walk_group<false, QUAD, false, false, false>(A, G, mac_thr, rec_thr, -1, wsm, blo, bhi, g, tg,
-                                                           f2_pack(e * e, e * e), acc, a2, a3, -1.f);
+                                                           f2_pack(e * e, e * e), acc, Part{0, 0, -1}, a2, a3, -1.f);
             if (!ok) {
                 if (lane == 0) latch_err(A.st, kErrStack);
                 continue;
@@ -861,16 +960,27 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
             }
             continue;
         }
-        // ---- a group of the tree, in queue order (skipped when the mask says none of its stars is active)
-        const int gk = A.order ? A.order[gi - A.n_extra] : gi - A.n_extra;
+        // ---- a part of a group's walk, in queue order (skipped when the mask says none of its stars is active)
+        gi -= A.n_extra;
+        const int gk = A.order ? A.order[gi] : gi / A.parts;
         if (A.gact && !A.gact[gk]) continue;
+        const int q = A.order ? A.opart[gi] : gi % A.parts;
         const GroupRec grp = load_group(A.groups, gk);
         if (grp.first < 0 || grp.count < 1 || grp.count > kMaxGroup || grp.first + grp.count > A.n) {
             if (lane == 0) latch_err(A.st, kErrStack);
             continue;
         }
-        const int mg = member_of(A.moff, A.M, grp.first);
-        const TreeGeo G = tree_geo(A, mg);
+        Part part;
+        TreeGeo G;
+        {
+            const int mg = member_of(A.moff, A.M, grp.first);
+            const int P = parts_of_group(A.parts, grp.count);
+            if (q >= P) continue;
+            part = part_of(q, P, A.moff[mg], A.moff[mg + 1] - A.moff[mg], A.n_leaf);
+            G = tree_geo(A, mg);
+            __syncwarp();
+            if (lane == 0) item[wib] = Item{gk, grp.first, grp.count, mg, q, P};
+        }
         if (G.root < 0) {
             if (lane == 0) latch_err(A.st, kErrStack);
             continue;
@@ -879,19 +989,19 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
         float g[3];
         box_centre(blo, bhi, G.lo, G.unit, g);
         // p target pairs (stars 2t, 2t + 1), k lanes per pair
-        const int s = grp.count, p = (s + 1) >> 1, k = 32 / p;
         Tgt tg;
         {
+            const int s = grp.count, p = (s + 1) >> 1, k = 32 / p;
             const int t = lane % p, sub = lane / p;
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
+            for (int h = 0; h < 2; h++) {
                 // an odd group's last pair repeats its star; those sums are not used
-                const float4 pq = __ldg(&A.pos[grp.first + min(2 * t + q, s - 1)]);
+                const float4 pq = __ldg(&A.pos[grp.first + min(2 * t + h, s - 1)]);
                 // minus the star's position relative to g (exact: FP32 negation)
                 const float nx = -(pq.x - g[0]), ny = -(pq.y - g[1]), nz = -(pq.z - g[2]);
-                tg.nx[q] = f2_pack(nx, nx);
-                tg.ny[q] = f2_pack(ny, ny);
-                tg.nz[q] = f2_pack(nz, nz);
+                tg.nx[h] = f2_pack(nx, nx);
+                tg.ny[h] = f2_pack(ny, ny);
+                tg.nz[h] = f2_pack(nz, nz);
             }
             tg.j0 = (sub < k) ? sub : (1 << 20);  // lanes beyond k p take no list pairs
             tg.k = k;
@@ -901,7 +1011,7 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
         float K = -1.f;
         if (REL) {
             float am = __int_as_float(0x7f800000);
-            for (int i = lane; i < s; i += 32) {
+            for (int i = lane; i < grp.count; i += 32) {
                 // |a| = sqrt((x x + y y) + z z) in FP32, one rounding per operation, as the oracle takes it
                 const int j = A.perm[grp.first + i];
                 const float x = A.arx[j], y = A.ary[j], z = A.arz[j];
@@ -910,27 +1020,43 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
             for (int o = 16; o > 0; o >>= 1) am = fminf(am, __shfl_xor_sync(0xffffffffu, am, o));
             if (am > 0.f) K = __fmul_rn(__fmul_rn(A.rel_alpha, am), __fmul_rn(G.unit, G.unit));
         }
-        bool ok = walk_group<SOFT, QUAD, REC, REL, SPL>(A, G, mac_thr, rec_thr, gk, wsm, blo, bhi, g, tg,
-                                                   f2_pack(A.eps2, A.eps2), acc, a2, a3, K);
-        if (!ok) {
-            if (lane == 0) latch_err(A.st, kErrStack);
-            continue;
+        clear_acc(accw);
+        const bool ok = walk_group<SOFT, QUAD, REC, REL, SPL>(A, G, mac_thr, rec_thr, gk, wsm, blo, bhi, g, tg,
+                                                         f2_pack(A.eps2, A.eps2), acc, part, a2, a3, K);
+        if (!ok && lane == 0) latch_err(A.st, kErrStack);
+        // (what the end of the item needs is read again: the walk has no registers to keep it)
+        const Item it = item[wib];
+        const int s = it.count, p = (s + 1) >> 1, k = 32 / p, P = it.P, mg = it.member, first = it.first;
+        if (ok && lane == 0) {
+            atomicAdd(&A.st->walk.n_p2p, (unsigned long long)a2 * s);
+            atomicAdd(&A.st->walk.n_m2p, (unsigned long long)a3 * s);
         }
-        np2p += a2 * (unsigned long long)s;
-        nm2p += a3 * (unsigned long long)s;
         Acc tots[2];
         combine_shares(accw, s, p, k, tots);
-        const float cost = (float)a2 + 2.5f * (float)a3;   // list pairs, a cell costing ~2.5 stars
+        if (P > 1) {
+            // the part's sums; the warp that finishes the group's last part adds
+            // them up. Every part has read its stars' references by then.
+            float4 *slot = A.partial + first;
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+                if (lane + 32 * h < s) slot[(int64_t)it.q * A.n + lane + 32 * h] = part_sum(tots[h]);
+            if (!last_part(A.garrive + it.group, P)) continue;
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+                if (lane + 32 * h < s) tots[h] = add_parts(slot + lane + 32 * h, A.n, P);
+        }
+        if (!ok) continue;
+        const float cost = P * ((float)a2 + 2.5f * (float)a3);   // list pairs, a cell costing ~2.5 stars
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int i = lane + 32 * h;
             if (i >= s) continue;
             Acc &tot = tots[h];
-            const float4 ps = __ldg(&A.pos[grp.first + i]);
+            const float4 ps = __ldg(&A.pos[first + i]);
             // the star's own pair was evaluated at r = 0: remove its -m/eps (the product
             // rounded on its own, as in the pair, so that the two cancel exactly)
             if (SOFT) tot.ph += __fmul_rn(ps.w, rsqrtf(A.eps2));
-            int o = A.perm[grp.first + i];
+            int o = A.perm[first + i];
             if (A.n_extra > 0) extra_terms(A, ps.x, ps.y, ps.z, A.eps_star, -1, mg, tot, !(A.xq_skip && A.xq_skip[o]));
             A.ax[o] = tot.ax + tot.cx;
             A.ay[o] = tot.ay + tot.cy;
@@ -939,31 +1065,38 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
             A.scost[o] = cost;
         }
     }
-    if (lane == 0) {
-        atomicAdd(&A.st->n_p2p, np2p);
-        atomicAdd(&A.st->n_m2p, nm2p);
-    }
 }
 
 // ---------------------------------------------------------------------------
-// Queue order of the groups: most expensive first (longest-processing-time
-// first: the walk's tail then holds the cheapest groups). The estimate is the
-// list cost the last walk recorded for the group's first star, if that walk
-// covered the same number of stars (st->cost_n); otherwise the volume of the
-// group's box, smallest first (small boxes sit in dense regions with long
-// lists). Groups are bucketed by log2 of the estimate (1/16 steps); the
-// order within a bucket is unspecified. The forces do not depend on it.
+// Queue order of the work items: most expensive first (longest-processing-time
+// first: the walk's tail then holds the cheapest ones). The estimate is the
+// list cost the last walk recorded for the group's first star, divided by the
+// group's parts, if that walk covered the same number of stars (st->cost_n);
+// otherwise the volume of the group's box, smallest first (small boxes sit in
+// dense regions with long lists). Groups are bucketed by log2 of the estimate
+// (1/16 steps), all parts of a group together; the order within a bucket is
+// unspecified. The forces do not depend on it.
 constexpr int kOrderBins = 1024;   // the workspace's obins holds this many
-constexpr int kOrderMinStars = 1 << 17;   // smaller systems walk their groups in build order
+// Smaller systems walk their items in build order: the three launches cost more
+// than the balance gives (walk of 16000 stars 150 us ordered or not, 65536 stars
+// 562 -> 543 us, 100003 stars in groups of 32 957 -> 892 us).
+constexpr int kOrderMinStars = 1 << 15;
 
-__device__ __forceinline__ int order_bin(const int4 *groups, const int *perm, const float *scost, int n, bool hist,
-                                         int g) {
-    const GroupRec r = load_group(groups, g);
+struct OrderArgs {
+    const int4 *groups;
+    const int *perm;
+    const float *scost;
+    int parts, n;
+};
+
+__device__ __forceinline__ int order_bin(const OrderArgs &A, bool hist, int g, int &P) {
+    const GroupRec r = load_group(A.groups, g);
+    const int first = min(max(r.first, 0), A.n - 1);
+    P = parts_of_group(A.parts, max(r.count, 1));
     float lv;
     if (hist) {
-        const int first = min(max(r.first, 0), n - 1);
         // any stored value is a finite estimate >= 1 here (NaN -> 1)
-        const float c = fminf(fmaxf(scost[perm[first]], 1.f), 1e30f);
+        const float c = fminf(fmaxf(A.scost[A.perm[first]] / P, 1.f), 1e30f);
         lv = 64.f - log2f(c);   // descending cost (a cost above 2^64 shares the first bin)
     } else {
         lv = log2f((float)max(r.hi[0] - r.lo[0], 1)) + log2f((float)max(r.hi[1] - r.lo[1], 1)) +
@@ -972,15 +1105,15 @@ __device__ __forceinline__ int order_bin(const int4 *groups, const int *perm, co
     return min(max((int)(16.f * lv), 0), kOrderBins - 1);
 }
 
-// (A) each group's bin, and the bin counts (bins zeroed before)
-__global__ void group_bins_k(const int4 *groups, DevState *st, const int *perm, const float *scost, int n, int *gbin,
-                             int *bins) {
+// (A) each group's bin (and its parts), and the bins' item counts (bins zeroed before)
+__global__ void group_bins_k(OrderArgs A, const DevState *st, int *gbin, int *bins) {
     const int ng = st->ngroup;
-    const bool hist = st->cost_n == n;
+    const bool hist = st->cost_n == A.n;
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
-        const int b = order_bin(groups, perm, scost, n, hist, g);
-        gbin[g] = b;
-        atomicAdd(&bins[b], 1);
+        int P;
+        const int b = order_bin(A, hist, g, P);
+        gbin[g] = b * (2 * kMaxParts) + P;
+        atomicAdd(&bins[b], P);
     }
 }
 
@@ -1010,14 +1143,21 @@ __global__ void __launch_bounds__(kOrderBins) group_bins_scan_k(DevState *st, in
     }
     __syncthreads();
     bins[t] = incl - v + wsum[w];
+    if (t == kOrderBins - 1) st->walk.nitem = incl + wsum[w];
     if (t == 0) st->cost_n = n;
 }
 
-// (C) each group to its place: order[next free slot of its bin] = g
-__global__ void group_scatter_k(const DevState *st, const int *gbin, int *bins, int *order) {
+// (C) each group's items to the next free slots of its bin
+__global__ void group_scatter_k(const DevState *st, const int *gbin, int *bins, int *order, uint8_t *opart) {
     const int ng = st->ngroup;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x)
-        order[atomicAdd(&bins[gbin[g]], 1)] = g;
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
+        const int b = gbin[g], P = b % (2 * kMaxParts);
+        const int at = atomicAdd(&bins[b / (2 * kMaxParts)], P);
+        for (int q = 0; q < P; q++) {
+            order[at + q] = g;
+            opart[at + q] = (uint8_t)q;
+        }
+    }
 }
 
 // MAC thresholds: the smallest integer D with fl(theta^2 * D) > s^2 (FP64,
@@ -1042,15 +1182,24 @@ MacTable mac_table(float theta) {
 
 template <bool SOFT, bool QUAD, bool REC, bool REL = false, bool SPL = false>
 static cudaError_t launch_walk(rv_ctx *c, const WalkArgs &A, cudaStream_t s) {
-    size_t smem = warp_smem_bytes(A.tile) * kWalkWarps;
+    const size_t smem = warp_smem_bytes(A.tile) * kWalkWarps;
     auto kern = walk_tree_k<SOFT, QUAD, REC, REL, SPL>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWalkWarps * 32, smem);
-    if (e != cudaSuccess) return e;
-    // every warp of the launch has its stack spill area
-    int grid = std::min(std::max(1, per_sm) * c->num_sms, kStackSpillWarps / kWalkWarps);
+    // resident blocks, asked once per context and variant (the tile is the context's). The
+    // attribute is the function's, shared by all contexts: always the largest tile's need.
+    int &blocks = c->walk_blocks[(REL ? 8 : 0) + (REC ? 4 : (SPL ? 4 : 0) + (SOFT ? 2 : 0) + (QUAD ? 1 : 0))];
+    if (blocks == 0) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)warp_smem_bytes(256) * kWalkWarps);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWalkWarps * 32, smem);
+        if (e != cudaSuccess) return e;
+        // every warp of the launch has its stack spill area
+        blocks = std::min(std::max(1, per_sm) * c->num_sms, kStackSpillWarps / kWalkWarps);
+    }
+    // no more warps than work items: at most one a star
+    const int64_t items = c->n + A.n_extra;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (items + kWalkWarps - 1) / kWalkWarps));
     kern<<<grid, kWalkWarps * 32, smem, s>>>(A);
     count_launch(c);
     return cudaGetLastError();
@@ -1094,9 +1243,13 @@ rv_status tree_walk(rv_ctx *c, float theta, float eps_star, int n_extra, const f
     if (rec) A.rec = mac_table(rec->theta_rec);
     A.gact = gact;
     A.gstack = w.gstack;
-    // systems with fewer groups than resident walk warps gain nothing from an order
     A.order = c->n >= kOrderMinStars ? w.gorder : nullptr;
+    A.opart = w.gopart;
     A.scost = w.scost;
+    A.n_leaf = c->cfg.n_leaf;
+    A.parts = parts_of(c->n, c->cfg.group);
+    A.partial = w.gpartial;
+    A.garrive = w.garrive;
     const bool spline = c->cfg.softening == 1 && eps_star > 0.f;
     {
         const float h = 2.8f * eps_star;
@@ -1109,9 +1262,8 @@ rv_status tree_walk(rv_ctx *c, float theta, float eps_star, int n_extra, const f
     A.ary = rel ? rel->ry : nullptr;
     A.arz = rel ? rel->rz : nullptr;
     if (rel && rec) return set_err(c, RV_E_INVAL, "no pair record under the relative criterion");
-    // reset the work counter and statistics (next_group, n_p2p, n_m2p)
-    cudaError_t e = cudaMemsetAsync(&w.st->next_group, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&w.st->n_p2p, 0, 2 * sizeof(unsigned long long), s);
+    // reset the work counter and statistics
+    cudaError_t e = cudaMemsetAsync(&w.st->walk, 0, sizeof(w.st->walk), s);
     if (e != cudaSuccess) return cuda_check(c, e, "walk reset");
     if (c->n == 0 && n_extra == 0) return RV_OK;
     const bool quad = c->cfg.quadrupole != 0;
@@ -1143,9 +1295,9 @@ rv_status tree_walk(rv_ctx *c, float theta, float eps_star, int n_extra, const f
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 255) / 256, (int64_t)c->num_sms * 4));
         e = cudaMemsetAsync(bins, 0, sizeof(int) * kOrderBins, s);
         if (e != cudaSuccess) return cuda_check(c, e, "walk order");
-        group_bins_k<<<grid, 256, 0, s>>>(w.groups, w.st, w.perm, w.scost, (int)c->n, gbin, bins);
+        group_bins_k<<<grid, 256, 0, s>>>(OrderArgs{w.groups, w.perm, w.scost, A.parts, (int)c->n}, w.st, gbin, bins);
         group_bins_scan_k<<<1, kOrderBins, 0, s>>>(w.st, (int)c->n, bins);
-        group_scatter_k<<<grid, 256, 0, s>>>(w.st, gbin, bins, w.gorder);
+        group_scatter_k<<<grid, 256, 0, s>>>(w.st, gbin, bins, w.gorder, w.gopart);
         c->launches += 3;
     }
     if (spline) {
