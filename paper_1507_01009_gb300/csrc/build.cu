@@ -50,79 +50,138 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *smem_warp, int &
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of int32 (in place), length *d_len (<= nmax) or nmax
+// Single-pass scans over tiles ("decoupled look-back": Merrill & Garland 2016).
+// A block takes the next tile from a ticket counter, publishes its tile's sum,
+// adds up its predecessors' published words back to the nearest full prefix,
+// and publishes its own prefix. A tile's predecessors have always started (the
+// tickets are handed out in order), so every wait ends; waits are bounded all
+// the same, and a block that gives up latches RV_E_TIMEOUT and writes nothing.
+// A word holds its state in the top two bits (0: not there yet) and the count
+// below (counts stay under 2^30), so that one store publishes both.
 // ---------------------------------------------------------------------------
-__global__ void scan_reduce_k(const int *data, int64_t nmax, const int *d_len, int *partials) {
-    __shared__ int sw[8];
-    int64_t len = d_len ? min((int64_t)*d_len, nmax) : nmax;
-    int64_t base = (int64_t)blockIdx.x * kScanChunk;
-    int sum = 0;
-    for (int i = threadIdx.x; i < kScanChunk; i += 256) {
-        int64_t j = base + i;
-        if (j < len) sum += data[j];
-    }
-    int total;
-    block_exclusive_scan<256>(sum, sw, total);
-    if (threadIdx.x == 0) partials[blockIdx.x] = total;
+constexpr unsigned kLbSum = 1u << 30, kLbPrefix = 2u << 30, kLbCount = (1u << 30) - 1;
+constexpr int kLbSpins = 1 << 22;   // polls before a wait gives up (seconds)
+
+__device__ __forceinline__ unsigned lb_load(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void lb_store(unsigned *p, unsigned v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__global__ void scan_partials_k(int *partials, int nb, int *d_total) {
-    __shared__ int sw[32];
-    int carry = 0;
-    for (int b0 = 0; b0 < nb; b0 += 1024) {
-        int b = b0 + threadIdx.x;
-        int v = (b < nb) ? partials[b] : 0;
-        int total;
-        int ex = block_exclusive_scan<1024>(v, sw, total);
-        if (b < nb) partials[b] = carry + ex;
-        carry += total;
+// The sum of the tiles before `tile` (one word a tile), by one whole warp: 32
+// predecessors a step. Returns false if a wait gave up.
+__device__ __forceinline__ bool lb_sum_before(const unsigned *words, int tile, unsigned &sum) {
+    const int lane = threadIdx.x & 31;
+    sum = 0;
+    for (int hi = tile - 1; hi >= 0; hi -= 32) {
+        const int t = hi - lane;
+        unsigned w = t >= 0 ? lb_load(words + t) : kLbPrefix;   // before the first tile: a prefix of 0
+        for (int spin = 0; __any_sync(0xffffffffu, (w >> 30) == 0); spin++) {
+            if (spin > kLbSpins) return false;
+            if ((w >> 30) == 0) w = lb_load(words + t);
+        }
+        const unsigned pm = __ballot_sync(0xffffffffu, w & kLbPrefix);
+        const int stop = pm ? __ffs(pm) - 1 : 31;   // the nearest prefix ends the search
+        sum += __reduce_add_sync(0xffffffffu, lane <= stop ? w & kLbCount : 0u);
+        if (pm) break;
     }
-    if (threadIdx.x == 0 && d_total) *d_total = carry;
+    return true;
 }
 
-__global__ void scan_down_k(int *data, int64_t nmax, const int *d_len, const int *partials) {
-    __shared__ int sw[8];
-    int64_t len = d_len ? min((int64_t)*d_len, nmax) : nmax;
-    int64_t base = (int64_t)blockIdx.x * kScanChunk + threadIdx.x * 8;
+// Exclusive scan of int32 (in place), length *d_len (<= nmax) or nmax; the
+// total to *d_total if given. words, ticket: zero before the launch.
+__global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int *d_len, unsigned *words, int *ticket,
+                                              int *d_total, DevState *st) {
+    __shared__ int sw[8], stile;
+    __shared__ unsigned sbefore;
+    __shared__ bool sok;
+    if (threadIdx.x == 0) stile = atomicAdd(ticket, 1);
+    __syncthreads();
+    const int tile = stile;
+    const int64_t len = d_len ? min((int64_t)*d_len, nmax) : nmax;
+    const int64_t base = (int64_t)tile * kScanChunk + threadIdx.x * 8;
     int v[8], s = 0;
+    if (base + 8 <= len) {   // the tile's start is 32-byte aligned
+        const int4 a = *reinterpret_cast<const int4 *>(data + base), b = *reinterpret_cast<const int4 *>(data + base + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        int64_t j = base + k;
-        v[k] = (j < len) ? data[j] : 0;
-        s += v[k];
+        for (int k = 0; k < 8; k++) v[k] = (base + k < len) ? data[base + k] : 0;
     }
+#pragma unroll
+    for (int k = 0; k < 8; k++) s += v[k];
     int total;
-    int ex = block_exclusive_scan<256>(s, sw, total) + partials[blockIdx.x];
+    const int ex0 = block_exclusive_scan<256>(s, sw, total);
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) lb_store(words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
+        unsigned before = 0;
+        const bool ok = lb_sum_before(words, tile, before);
+        if (threadIdx.x == 0) {
+            if (ok && tile) lb_store(words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
+            if (!ok) latch_err(st, kErrTimeout);
+            sbefore = before;
+            sok = ok;
+            if (ok && d_total && tile == (int)gridDim.x - 1) *d_total = (int)before + total;
+        }
+    }
+    __syncthreads();
+    if (!sok) return;
+    int ex = ex0 + (int)sbefore;
+    int o[8];
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        int64_t j = base + k;
-        if (j < len) data[j] = ex;
+        o[k] = ex;
         ex += v[k];
     }
+    if (base + 8 <= len) {
+        *reinterpret_cast<int4 *>(data + base) = make_int4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<int4 *>(data + base + 4) = make_int4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (base + k < len) data[base + k] = o[k];
+    }
 }
 
-rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, const int *d_len, int *d_total, cudaStream_t s) {
+static rv_status scan_launch(rv_ctx *c, int *data, int64_t nmax, int *d_total, unsigned *words, int *ticket,
+                             cudaStream_t s) {
+    scan_k<<<ceil_div(nmax, kScanChunk), 256, 0, s>>>(data, nmax, nullptr, words, ticket, d_total, c->w.st);
+    count_launch(c);
+    return cuda_check(c, cudaGetLastError(), "scan");
+}
+
+rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s) {
     if (nmax <= 0) {
         if (d_total) return cuda_check(c, cudaMemsetAsync(d_total, 0, sizeof(int), s), "scan memset");
         return RV_OK;
     }
-    int nb = ceil_div(nmax, kScanChunk);
-    scan_reduce_k<<<nb, 256, 0, s>>>(data, nmax, d_len, c->w.partials);
-    count_launch(c);
-    scan_partials_k<<<1, 1024, 0, s>>>(c->w.partials, nb, d_total);
-    count_launch(c);
-    scan_down_k<<<nb, 256, 0, s>>>(data, nmax, d_len, c->w.partials);
-    count_launch(c);
-    return cuda_check(c, cudaGetLastError(), "scan");
+    // ticket and words side by side: one clear
+    unsigned *z = c->w.lb + kLbScan;
+    rv_status r = cuda_check(c, cudaMemsetAsync(z, 0, sizeof(unsigned) * (1 + (size_t)ceil_div(nmax, kScanChunk)), s),
+                             "scan");
+    if (r != RV_OK) return r;
+    return scan_launch(c, data, nmax, d_total, z + 1, reinterpret_cast<int *>(z), s);
 }
 
 // ---------------------------------------------------------------------------
 // bounding cube
 // ---------------------------------------------------------------------------
-// Blocks (bx, m): member m's stars, strided by bpm blocks.
-__global__ void bounds_partial_k(const int64_t *moff, int bpm, const float *x, const float *y, const float *z,
-                                 float *part) {
+// Blocks (bx, m): member m's stars, strided by bpm blocks; the last block of a
+// member to finish reduces the blocks' partials: min per axis; L = max_a (max_a
+// - min_a) with FP64 differences; scale = 2^21 / L (min and max are exact, so
+// the order is free). The first kernel of a build, it also clears the words the
+// later ones count in (zero[nzero]) and the member roots.
+__global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, const float *x, const float *y,
+                                                const float *z, float *part, int *arrive, double *mbounds,
+                                                DevState *st, unsigned *zero, int64_t nzero, int *mroot) {
     const int m = blockIdx.y;
+    const int64_t nthr = (int64_t)gridDim.x * gridDim.y * 256;
+    const int64_t tid = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.x;
+    for (int64_t i = tid; i < nzero; i += nthr) zero[i] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) mroot[m] = -1;
     const int64_t s = moff[m], e = moff[m + 1];
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int64_t i = s + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (int64_t)bpm * blockDim.x) {
@@ -133,42 +192,44 @@ __global__ void bounds_partial_k(const int64_t *moff, int bpm, const float *x, c
             hi[a] = fmaxf(hi[a], v[a]);
         }
     }
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-    }
     __shared__ float sh[8][6];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    auto warp_minmax = [&]() {
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            for (int o = 16; o > 0; o >>= 1) {
+                lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+                hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+            }
+    };
+    warp_minmax();
     if (lane == 0)
         for (int a = 0; a < 3; a++) { sh[wid][a] = lo[a]; sh[wid][3 + a] = hi[a]; }
     __syncthreads();
     if (threadIdx.x < 6) {
         float r = sh[0][threadIdx.x];
-        for (int w = 1; w < (int)(blockDim.x >> 5); w++)
+        for (int w = 1; w < 8; w++)
             r = (threadIdx.x < 3) ? fminf(r, sh[w][threadIdx.x]) : fmaxf(r, sh[w][threadIdx.x]);
         part[6 * ((int64_t)m * bpm + blockIdx.x) + threadIdx.x] = r;
+        __threadfence();
     }
-}
-
-// One warp per member: min per axis; L = max_a (max_a - min_a) with FP64
-// differences; scale = 2^21 / L (min and max are exact, so order is free).
-__global__ void bounds_final_k(int bpm, const float *part, double *mbounds, DevState *st) {
-    const int m = blockIdx.x;
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int b = threadIdx.x; b < bpm; b += 32)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(arrive + m, 1) == bpm - 1;
+        if (last) arrive[m] = 0;   // ready for the next build
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last || wid != 0) return;
+    for (int a = 0; a < 3; a++) { lo[a] = INFINITY; hi[a] = -INFINITY; }
+    for (int b = lane; b < bpm; b += 32)
         for (int a = 0; a < 3; a++) {
-            lo[a] = fminf(lo[a], part[6 * ((int64_t)m * bpm + b) + a]);
-            hi[a] = fmaxf(hi[a], part[6 * ((int64_t)m * bpm + b) + 3 + a]);
+            lo[a] = fminf(lo[a], __ldcg(&part[6 * ((int64_t)m * bpm + b) + a]));
+            hi[a] = fmaxf(hi[a], __ldcg(&part[6 * ((int64_t)m * bpm + b) + 3 + a]));
         }
-    for (int a = 0; a < 3; a++)
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-    if (threadIdx.x != 0) return;
+    warp_minmax();
+    if (lane != 0) return;
     double out[5];
     double L = 0.0;
     for (int a = 0; a < 3; a++) {
@@ -271,190 +332,321 @@ __device__ __forceinline__ uint32_t grid_coord_fast(float v, const GridAxis &g) 
     return grid_coord(v, g.lo, g.scale);
 }
 
+// Digit counts of one key per lane (ok: the lane has one) into the block's
+// [passes][kSortBins] counters. The high digits of a centrally concentrated
+// system hold few values: there the lanes of a warp with one digit add once.
+template <int PASSES>
+__device__ __forceinline__ void count_digits(uint64_t k, bool ok, int *h) {
+    const unsigned lt = lanemask_lt();
+#pragma unroll
+    for (int p = 0; p < PASSES; p++) {
+        const int d = (int)(k >> (p * kSortBits)) & (kSortBins - 1);
+        if (p >= 3) {
+            const unsigned peers = __match_any_sync(0xffffffffu, ok ? d : -1);
+            if (ok && (peers & lt) == 0) atomicAdd(&h[p * kSortBins + d], __popc(peers));
+        } else if (ok) {
+            atomicAdd(&h[p * kSortBins + d], 1);
+        }
+    }
+}
+
 // Blocks (bx, m): member m's stars with member m's bounding cube. Each star's
 // (x, y, z, m) is also packed into one float4 (caller order), so that the
 // gather into key order reads one 16-byte record per star instead of four
-// scattered 4-byte values (each costing a 32-byte sector).
-__global__ void keys_k(const int64_t *moff, int bpm, const float *x, const float *y, const float *z,
-                       const float *mass, const double *mbounds, uint64_t *key, float4 *xyzm) {
+// scattered 4-byte values (each costing a 32-byte sector). The digit counts of
+// all sort passes are taken here, where the keys are in registers (the sort
+// then reads them only to move them), and the first pass's look-back words are cleared.
+__global__ void __launch_bounds__(256) keys_k(const int64_t *moff, int bpm, const float *x, const float *y,
+                                              const float *z, const float *mass, const double *mbounds, uint64_t *key,
+                                              float4 *xyzm, unsigned *ghist, uint4 *words, int64_t nwords4) {
+    __shared__ int h[kKeyPasses * kSortBins];
+    for (int b = threadIdx.x; b < kKeyPasses * kSortBins; b += 256) h[b] = 0;
+    const int64_t nthr = (int64_t)gridDim.x * gridDim.y * 256;
+    for (int64_t i = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < nwords4; i += nthr)
+        words[i] = make_uint4(0, 0, 0, 0);
     const int m = blockIdx.y;
     const double sc = mbounds[5 * m + 4];
     const GridAxis gx = grid_axis(mbounds[5 * m], sc), gy = grid_axis(mbounds[5 * m + 1], sc),
                    gz = grid_axis(mbounds[5 * m + 2], sc);
     const int64_t s = moff[m], e = moff[m + 1];
-    for (int64_t i = s + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (int64_t)bpm * blockDim.x) {
-        const float xi = x[i], yi = y[i], zi = z[i];
-        uint64_t k = spread3(grid_coord_fast(xi, gx)) | (spread3(grid_coord_fast(yi, gy)) << 1) |
-                     (spread3(grid_coord_fast(zi, gz)) << 2);
-        key[i] = k;
-        xyzm[i] = make_float4(xi, yi, zi, mass[i]);
+    __syncthreads();
+    const int64_t w0 = s + (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31);   // the warp's first star
+    for (int64_t b = w0; b < e; b += (int64_t)bpm * 256) {
+        const int64_t i = b + (threadIdx.x & 31);
+        const bool ok = i < e;
+        uint64_t k = 0;
+        if (ok) {
+            const float xi = x[i], yi = y[i], zi = z[i];
+            k = spread3(grid_coord_fast(xi, gx)) | (spread3(grid_coord_fast(yi, gy)) << 1) |
+                (spread3(grid_coord_fast(zi, gz)) << 2);
+            key[i] = k;
+            xyzm[i] = make_float4(xi, yi, zi, mass[i]);
+        }
+        count_digits<kKeyPasses>(k, ok, h);
     }
+    __syncthreads();
+    for (int b = threadIdx.x; b < kKeyPasses * kSortBins; b += 256)
+        if (h[b]) atomicAdd(&ghist[b], (unsigned)h[b]);
 }
 
 // ---------------------------------------------------------------------------
-// stable LSD radix sort of (key, index), 9-bit digits
+// stable LSD radix sort of (key, index), 9-bit digits, one kernel a pass
 // ---------------------------------------------------------------------------
-// Digit of element j: 9 key bits from `shift`, or (member pass) the member of
-// its caller index, which groups the members while keeping each one's order.
-__device__ __forceinline__ int sort_digit(const uint64_t *key, const int *idx, int64_t j, int shift,
-                                          const int64_t *moff, int M) {
-    if (moff) return member_of(moff, M, (int64_t)idx[j]);
-    return (int)((key[j] >> shift) & (kSortBins - 1));
-}
-
-__global__ void __launch_bounds__(kSortThreads) sort_upsweep_k(int64_t n, const uint64_t *key, const int *idx,
-                                                               int shift, const int64_t *moff, int M, int ntiles,
-                                                               int *hist) {
-    __shared__ int h[kSortBins];
-    for (int b = threadIdx.x; b < kSortBins; b += kSortThreads) h[b] = 0;
+// The digit counts of `passes` passes of a key array (sorts other than the build's).
+__global__ void __launch_bounds__(256) sort_hist_k(int64_t n, const uint64_t *key, int passes, unsigned *ghist) {
+    __shared__ int h[4 * kSortBins];
+    for (int b = threadIdx.x; b < 4 * kSortBins; b += 256) h[b] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kSortTile;
-    int d[kSortItems];
-#pragma unroll
-    for (int k = 0; k < kSortItems; k++) {   // the tile's loads first
-        const int64_t j = base + k * kSortThreads + threadIdx.x;
-        d[k] = j < n ? sort_digit(key, idx, j, shift, moff, M) : -1;
+    for (int64_t b = (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31); b < n; b += (int64_t)gridDim.x * 256) {
+        const int64_t i = b + (threadIdx.x & 31);
+        count_digits<4>(i < n ? key[i] : 0ull, i < n, h);
     }
-#pragma unroll
-    for (int k = 0; k < kSortItems; k++)
-        if (d[k] >= 0) atomicAdd(&h[d[k]], 1);
     __syncthreads();
-    for (int b = threadIdx.x; b < kSortBins; b += kSortThreads) hist[(int64_t)b * ntiles + blockIdx.x] = h[b];
+    for (int b = threadIdx.x; b < passes * kSortBins; b += 256)
+        if (h[b]) atomicAdd(&ghist[b], (unsigned)h[b]);
 }
 
-// Each warp ranks 256 consecutive keys in 8 rounds of 32 (warp-private digit
-// counters), so the in-tile order is (warp, round, lane) = input order and the
-// sort is stable. The ranked tile is then staged in shared memory in digit
-// order and written out from there: consecutive threads write consecutive
-// slots of a digit's output run (coalesced), instead of each thread writing
-// its own element straight to a scattered destination.
-__global__ void __launch_bounds__(kSortThreads) sort_downsweep_k(int64_t n, const uint64_t *key_in,
-                                                                 const int *idx_in, int shift, const int64_t *moff,
-                                                                 int M, int ntiles, const int *hist,
-                                                                 uint64_t *key_out, int *idx_out) {
-    constexpr int NW = kSortThreads / 32;
-    __shared__ unsigned short cnt[NW][kSortBins];
-    __shared__ int gbase[kSortBins];
-    __shared__ int lstart[kSortBins];            // first staged slot of each digit
-    __shared__ uint64_t skey[kSortTile];
-    __shared__ int sidx[kSortTile];
-    __shared__ unsigned short sdig[kSortTile];
-    __shared__ int sw[NW];
+// One pass: the digit of element j is 9 key bits from `shift`, or (moff: the
+// member pass) the member of its caller index, which groups the members while
+// keeping each one's order. A block takes the next tile of TILE = 256 ITEMS
+// elements. Each warp ranks its consecutive keys in ITEMS rounds of 32
+// (warp-private digit counters), so the in-tile order is (warp, round, lane) =
+// input order and the sort is stable; thread t owns digits 2t and 2t + 1,
+// publishes their counts in the tile, and looks back for the counts before it
+// (the words of tile t: words[t][kSortBins]); the tile is staged in shared
+// memory in digit order and written out from there, consecutive threads to
+// consecutive slots of a digit's output run. The digits' first slots are the
+// exclusive scan of the digit counts `ghist` (or the members' offsets). The last
+// pass also gathers the stars (pos). words_next: the next pass's words, cleared
+// here tile by tile (null: none).
+//
+// One launch a pass and 24 B an element, against five launches and 32 B for a
+// count, a three-kernel scan and a move: seven passes 190 -> 73 us on 100003
+// stars, where launches and latency count. Large sorts are bound by the ranking
+// rounds and the short output runs (512 digits a tile of 4096: 8 elements a run;
+// 2^24 elements 260 us a pass, 1.5 TB/s).
+template <int ITEMS>
+struct SortSmem {
+    unsigned short cnt[kSortThreads / 32][kSortBins];
+    int gbase[kSortBins];                        // first output slot of each digit for this tile
+    int lstart[kSortBins];                       // first staged slot of each digit
+    uint64_t key[kSortThreads * ITEMS];
+    int idx[kSortThreads * ITEMS];
+    unsigned short dig[kSortThreads * ITEMS];
+    int sw[kSortThreads / 32];
+    int tile;
+};
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uint64_t *key_in, const int *idx_in,
+                                                            int shift, const int64_t *moff, int M,
+                                                            const unsigned *ghist, int *ticket, unsigned *words,
+                                                            unsigned *words_next, uint64_t *key_out, int *idx_out,
+                                                            const float4 *xyzm, float4 *pos, DevState *st) {
+    constexpr int NW = kSortThreads / 32, TILE = kSortThreads * ITEMS;
+    static_assert(kSortBins == 2 * kSortThreads, "a thread owns two digits");
+    extern __shared__ __align__(16) char sort_smem[];
+    SortSmem<ITEMS> &S = *reinterpret_cast<SortSmem<ITEMS> *>(sort_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int b = lane; b < kSortBins; b += 32) cnt[wid][b] = 0;
-    for (int b = threadIdx.x; b < kSortBins; b += kSortThreads)
-        gbase[b] = hist[(int64_t)b * ntiles + blockIdx.x];
-    __syncwarp();
-    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-    const int64_t base = tile0 + wid * (32 * kSortItems);
-    uint64_t kk[kSortItems];
-    int ix[kSortItems], digit[kSortItems], rank[kSortItems];
+    if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1);
+    for (int b = lane; b < kSortBins / 2; b += 32) reinterpret_cast<unsigned *>(S.cnt[wid])[b] = 0;
+    __syncthreads();
+    const int tile = S.tile;
+    const int64_t tile0 = (int64_t)tile * TILE;
+    const int64_t base = tile0 + wid * (32 * ITEMS);
+    const int d0 = 2 * threadIdx.x;   // this thread's digits
+    if (words_next) *reinterpret_cast<uint2 *>(words_next + (int64_t)tile * kSortBins + d0) = make_uint2(0, 0);
+    uint64_t kk[ITEMS];
+    int ix[ITEMS], digit[ITEMS], rank[ITEMS];
     // every load of the tile first, so that their latencies overlap (the
     // ranking rounds below synchronise the warp)
 #pragma unroll
-    for (int r = 0; r < kSortItems; r++) {
+    for (int r = 0; r < ITEMS; r++) {
         const int64_t j = base + r * 32 + lane;
         const bool ok = j < n;
         kk[r] = ok ? key_in[j] : 0ull;
         ix[r] = ok ? (idx_in ? idx_in[j] : (int)j) : 0;
     }
+    // the digits' counts in the whole input (the member pass: the members' offsets)
+    int g0 = 0, g1 = 0;
+    if (!moff) {
+        g0 = (int)__ldg(ghist + d0);
+        g1 = (int)__ldg(ghist + d0 + 1);
+    }
 #pragma unroll
-    for (int r = 0; r < kSortItems; r++) {
+    for (int r = 0; r < ITEMS; r++) {
         const int64_t j = base + r * 32 + lane;
         int d = kSortBins;
         if (j < n) d = moff ? member_of(moff, M, (int64_t)ix[r]) : (int)((kk[r] >> shift) & (kSortBins - 1));
         digit[r] = d;
         unsigned peers = __match_any_sync(0xffffffffu, d);
-        int before = (d < kSortBins) ? cnt[wid][d] : 0;
+        int before = (d < kSortBins) ? S.cnt[wid][d] : 0;
         rank[r] = before + __popc(peers & lanemask_lt());
         __syncwarp();
-        if (d < kSortBins && lane == __ffs(peers) - 1) cnt[wid][d] = (unsigned short)(before + __popc(peers));
+        if (d < kSortBins && lane == __ffs(peers) - 1) S.cnt[wid][d] = (unsigned short)(before + __popc(peers));
         __syncwarp();
     }
     __syncthreads();
     // per digit: the warps' counts become offsets within the digit's run of this tile
-    static_assert(kSortBins % kSortThreads == 0, "each thread owns whole digits");
-    int tot[kSortBins / kSortThreads];
+    int tot0 = 0, tot1 = 0;
 #pragma unroll
-    for (int q = 0; q < kSortBins / kSortThreads; q++) {
-        const int b = threadIdx.x * (kSortBins / kSortThreads) + q;
-        int run = 0;
-        for (int w = 0; w < NW; w++) {
-            int t = cnt[w][b];
-            cnt[w][b] = (unsigned short)run;
-            run += t;
-        }
-        tot[q] = run;
+    for (int w = 0; w < NW; w++) {
+        ushort2 *q = reinterpret_cast<ushort2 *>(&S.cnt[w][d0]);
+        const ushort2 t = *q;
+        *q = make_ushort2((unsigned short)tot0, (unsigned short)tot1);
+        tot0 += t.x;
+        tot1 += t.y;
     }
-    // digit runs in digit order: exclusive scan of the tile's digit totals
-    {
-        int mine = 0;
+    unsigned *mine = words + (int64_t)tile * kSortBins + d0;
+    const unsigned state = tile ? kLbSum : kLbPrefix;
+    lb_store(mine, state | (unsigned)tot0);
+    lb_store(mine + 1, state | (unsigned)tot1);
+    // digit runs in digit order: exclusive scans of the tile's totals and of the whole input's
+    int total;
+    const int ex = block_exclusive_scan<kSortThreads>(tot0 + tot1, S.sw, total);
+    S.lstart[d0] = ex;
+    S.lstart[d0 + 1] = ex + tot0;
+    int first0, first1;
+    if (moff) {
+        first0 = d0 < M ? (int)moff[d0] : 0;
+        first1 = d0 + 1 < M ? (int)moff[d0 + 1] : 0;
+    } else {
+        const int gx = block_exclusive_scan<kSortThreads>(g0 + g1, S.sw, total);
+        first0 = gx;
+        first1 = gx + g0;
+    }
+    // counts of this thread's digits in the tiles before, four tiles' words in flight
+    bool fail = false;
+    unsigned b0 = 0, b1 = 0;
+    bool done0 = tile == 0, done1 = tile == 0;
+    for (int t = tile - 1, spin = 0; !(done0 && done1);) {
+        uint2 w[4];
 #pragma unroll
-        for (int q = 0; q < kSortBins / kSortThreads; q++) mine += tot[q];
-        int total;
-        int ex = block_exclusive_scan<kSortThreads>(mine, sw, total);
+        for (int q = 0; q < 4; q++) {
+            const unsigned *p = words + (int64_t)max(t - q, 0) * kSortBins + d0;
+            w[q].x = lb_load(p);
+            w[q].y = lb_load(p + 1);
+        }
+        int used = 0;
 #pragma unroll
-        for (int q = 0; q < kSortBins / kSortThreads; q++) {
-            lstart[threadIdx.x * (kSortBins / kSortThreads) + q] = ex;
-            ex += tot[q];
+        for (int q = 0; q < 4; q++) {
+            // in order, while every tile so far was there (tile 0's words are prefixes)
+            if (used == q && (done0 || (w[q].x >> 30)) && (done1 || (w[q].y >> 30))) {
+                used = q + 1;
+                if (!done0) {
+                    b0 += w[q].x & kLbCount;
+                    done0 = (w[q].x & kLbPrefix) != 0;
+                }
+                if (!done1) {
+                    b1 += w[q].y & kLbCount;
+                    done1 = (w[q].y & kLbPrefix) != 0;
+                }
+            }
+        }
+        t -= used;
+        if (used == 0 && ++spin > kLbSpins) {
+            fail = true;
+            break;
         }
     }
-    __syncthreads();
+    if (tile && !fail) {
+        lb_store(mine, kLbPrefix | ((b0 + (unsigned)tot0) & kLbCount));
+        lb_store(mine + 1, kLbPrefix | ((b1 + (unsigned)tot1) & kLbCount));
+    }
+    S.gbase[d0] = first0 + (int)b0 - ex;
+    S.gbase[d0 + 1] = first1 + (int)b1 - (ex + tot0);
+    if (__syncthreads_or(fail)) {   // a wait gave up: nothing is written
+        if (threadIdx.x == 0) latch_err(st, kErrTimeout);
+        return;
+    }
 #pragma unroll
-    for (int r = 0; r < kSortItems; r++) {
-        int64_t j = base + r * 32 + lane;
+    for (int r = 0; r < ITEMS; r++) {
+        const int64_t j = base + r * 32 + lane;
         if (j < n) {
             const int d = digit[r];
-            const int slot = lstart[d] + cnt[wid][d] + rank[r];
-            skey[slot] = kk[r];
-            sidx[slot] = ix[r];
-            sdig[slot] = (unsigned short)d;
+            const int slot = S.lstart[d] + S.cnt[wid][d] + rank[r];
+            S.key[slot] = kk[r];
+            S.idx[slot] = ix[r];
+            S.dig[slot] = (unsigned short)d;
         }
     }
     __syncthreads();
-    const int tn = (int)min((int64_t)kSortTile, n - tile0);
-    for (int t = threadIdx.x; t < tn; t += kSortThreads) {
-        const int d = sdig[t];
-        const int64_t dst = (int64_t)gbase[d] + (t - lstart[d]);
-        key_out[dst] = skey[t];
-        idx_out[dst] = sidx[t];
+    const int tn = (int)min((int64_t)TILE, n - tile0);
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+        const int t = r * kSortThreads + threadIdx.x;
+        if (t >= tn) break;
+        const int64_t dst = (int64_t)S.gbase[S.dig[t]] + t;
+        const int i = S.idx[t];
+        key_out[dst] = S.key[t];
+        idx_out[dst] = i;
+        if (pos) pos[dst] = __ldg(&xyzm[i]);
     }
 }
 
-rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, bool identity_idx,
-                     cudaStream_t s, bool member_pass) {
+// Items a thread (tile / 256): small sorts in small tiles (more blocks), large
+// ones in large tiles (longer output runs). Whole build in us with tiles of
+// 1024, 2048, 4096: 195, 189, 203 on 200001 stars, 300, 272, 261 on 2^19,
+// 473, 417, 387 on 2^20; 2^24: 3876 at 2048, 3820 at 4096.
+constexpr int64_t kSortN4 = 1 << 17, kSortN8 = 1 << 18;
+static int sort_items(int64_t n) { return n < kSortN4 ? 4 : n < kSortN8 ? 8 : 16; }
+
+int64_t sort_words(int64_t n_max) {
+    int64_t tiles = 1;
+    for (int64_t n : {std::min(n_max, kSortN4 - 1), std::min(n_max, kSortN8 - 1), n_max})
+        tiles = std::max<int64_t>(tiles, ceil_div(n, kSortThreads * sort_items(n)));
+    return tiles * kSortBins;
+}
+
+template <int ITEMS>
+static void sort_pass(rv_ctx *c, int64_t n, const uint64_t *ki, const int *ii, int shift, const int64_t *moff,
+                      const unsigned *ghist, int *ticket, unsigned *words, unsigned *next, uint64_t *ko, int *io,
+                      const float4 *xyzm, float4 *pos, cudaStream_t s) {
+    auto kern = sort_pass_k<ITEMS>;
+    if (sizeof(SortSmem<ITEMS>) > 48 * 1024)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem<ITEMS>));
+    kern<<<ceil_div(n, kSortThreads * ITEMS), kSortThreads, sizeof(SortSmem<ITEMS>), s>>>(
+        n, ki, ii, shift, moff, c->n_members, ghist, ticket, words, next, ko, io, xyzm, pos, c->w.st);
+    count_launch(c);
+}
+
+// Sorts key_a with identity indices; `counted`: the digit counts, tickets and
+// the first pass's words are set up already (the build's first kernels). With
+// pos, the stars xyzm are gathered into key order by the last pass.
+rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, cudaStream_t s, bool member_pass,
+                     bool counted, const float4 *xyzm, float4 *pos) {
     if (n <= 0) return RV_OK;
-    int ntiles = ceil_div(n, kSortTile);
-    uint64_t *kin = c->w.key_a, *kout = c->w.key_b;
-    int *iin = identity_idx ? nullptr : c->w.idx_a, *iout = c->w.idx_b;
-    const int M = c->n_members;
-    const int total = passes + ((member_pass && M > 1) ? 1 : 0);
+    Workspace &w = c->w;
+    const int items = sort_items(n);
+    unsigned *ghist = w.lb + kLbHist;
+    int *tickets = reinterpret_cast<int *>(w.lb + kLbTickets);
+    if (!counted) {
+        const int ntiles = ceil_div(n, kSortThreads * items);
+        rv_status r = cuda_check(c, cudaMemsetAsync(w.lb, 0, sizeof(unsigned) * kLbScan, s), "radix sort");
+        if (r == RV_OK)
+            r = cuda_check(c, cudaMemsetAsync(w.words[0], 0, sizeof(unsigned) * kSortBins * (size_t)ntiles, s), "radix sort");
+        if (r != RV_OK) return r;
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 1024), (int64_t)c->num_sms * 4));
+        sort_hist_k<<<grid, 256, 0, s>>>(n, w.key_a, passes, ghist);
+        count_launch(c);
+    }
+    uint64_t *kin = w.key_a, *kout = w.key_b;
+    int *iin = nullptr, *iout = w.idx_b;
+    const int total = passes + ((member_pass && c->n_members > 1) ? 1 : 0);
     for (int p = 0; p < total; p++) {
-        int shift = p * kSortBits;
-        const int64_t *moff = (p == passes) ? c->w.moff : nullptr;  // last pass: members
-        sort_upsweep_k<<<ntiles, kSortThreads, 0, s>>>(n, kin, iin, shift, moff, M, ntiles, c->w.hist);
-        count_launch(c);
-        rv_status st = exclusive_scan(c, c->w.hist, (int64_t)kSortBins * ntiles, nullptr, nullptr, s);
-        if (st != RV_OK) return st;
-        sort_downsweep_k<<<ntiles, kSortThreads, 0, s>>>(n, kin, iin, shift, moff, M, ntiles, c->w.hist, kout,
-                                                          iout);
-        count_launch(c);
+        const bool mem = p == passes, lastp = p + 1 == total;
+        auto run = items == 4 ? sort_pass<4> : items == 8 ? sort_pass<8> : sort_pass<16>;
+        run(c, n, kin, iin, p * kSortBits, mem ? w.moff : nullptr, mem ? nullptr : ghist + p * kSortBins, tickets + p,
+            w.words[p & 1], lastp ? nullptr : w.words[(p + 1) & 1], kout, iout, lastp ? xyzm : nullptr,
+            lastp ? pos : nullptr, s);
         // next pass reads what this one wrote
         uint64_t *tk = kin; kin = kout; kout = tk;
-        int *ti = (iin == nullptr) ? c->w.idx_a : iin;
+        int *ti = (iin == nullptr) ? w.idx_a : iin;
         iin = iout; iout = ti;
     }
     *keys = kin;
     *idx = iin;
     return cuda_check(c, cudaGetLastError(), "radix sort");
-}
-
-// ---------------------------------------------------------------------------
-// gather (x, y, z, m) into key order
-// ---------------------------------------------------------------------------
-__global__ void gather_k(int64_t n, const int *perm, const float4 *xyzm, float4 *pos) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        pos[i] = xyzm[perm[i]];
 }
 
 // ---------------------------------------------------------------------------
@@ -629,48 +821,93 @@ __global__ void __launch_bounds__(kTopoBlock) topo_write_k(int64_t n, const uint
 // [min q, max q + 1), q the star's de-interleaved key. Every star lies in its
 // group's box, so a cell the box-box test accepts passes the opening test for
 // each star of the group.
-// gcnt[c] = groups of cell c (0 unless c is a unit).
-__global__ void groups_count_k(const int4 *cbox, const int4 *clink, const int *cparent, int G, int U, int64_t cap,
-                               const DevState *st, int *gcnt) {
-    const int ncell = (int)min((int64_t)st->ncell, cap);
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-        const int4 lk = clink[c];
-        const int cnt = lk.w - lk.z;
-        bool unit;
-        if (cnt > U) {
-            unit = (lk.x == lk.y);   // an overfull leaf
-        } else if (cbox[c].w == 0) {
-            unit = true;             // a member's root
-        } else {
-            const int p = cparent[c];
-            unit = false;
-            if (p >= 0 && p < ncell) {
-                const int4 pl = clink[p];
-                unit = (pl.w - pl.z) > U;
-            }
+//
+// One pass over the cells in tiles of `tc` (<= 256) cells: a thread counts its
+// cell's groups, the block scans the counts and looks back for the groups of
+// the tiles before, and its warps take the tile's groups one by one. (A count, a
+// three-kernel scan and a writing pass whose warps took a unit's groups in turn:
+// 35 us on 100003 stars, hidden now behind the multipoles.)
+struct GroupArgs {
+    const uint64_t *skey;
+    const int4 *cbox, *clink;
+    const int *cparent;
+    int G, U, tc;
+    int64_t cap;
+    unsigned *words;   // look-back words, zero before the launch
+    int *ticket;
+    int4 *groups;
+    int *garrive;
+    DevState *st;
+};
+
+struct GroupSmem {
+    int ofs[256], first[256], end[256];   // per cell of the tile: its first group, its stars
+    int sw[8], tile;
+    unsigned before;
+    bool ok;
+};
+
+__device__ __forceinline__ int unit_groups(const GroupArgs &A, int c, int ncell, int4 &lk) {
+    lk = A.clink[c];
+    const int cnt = lk.w - lk.z;
+    bool unit = false;
+    if (cnt > A.U) {
+        unit = (lk.x == lk.y);   // an overfull leaf
+    } else if (A.cbox[c].w == 0) {
+        unit = true;             // a member's root
+    } else {
+        const int p = A.cparent[c];
+        if (p >= 0 && p < ncell) {
+            const int4 pl = A.clink[p];
+            unit = (pl.w - pl.z) > A.U;
         }
-        gcnt[c] = unit ? (cnt + G - 1) / G : 0;
     }
+    return unit ? (cnt + A.G - 1) / A.G : 0;
 }
 
-// One warp per unit cell: writes its runs with their boxes from the scanned
-// offsets gofs (exclusive prefix of gcnt).
-__global__ void groups_write_k(const uint64_t *skey, const int4 *clink, const int *gofs, const int *gcnt_total,
-                               int G, int64_t cap, const DevState *st, int4 *groups, int *garrive) {
-    const int lane = threadIdx.x & 31;
-    const int ncell = (int)min((int64_t)st->ncell, cap);
-    const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
-    for (int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < ncell; c += nw) {
-        const int g0 = gofs[c];
-        const int g1 = (c + 1 < ncell) ? gofs[c + 1] : *gcnt_total;
-        if (g1 <= g0) continue;
-        const int4 lk = clink[c];
-        for (int r = 0; r < g1 - g0; r++) {
-            const int first = lk.z + r * G;
-            const int cnt = min(G, lk.w - first);
+__device__ void write_groups(const GroupArgs &A, GroupSmem &S) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ncell = (int)min((int64_t)A.st->ncell, A.cap);
+    while (true) {
+        __syncthreads();
+        if (threadIdx.x == 0) S.tile = atomicAdd(A.ticket, 1);
+        __syncthreads();
+        const int tile = S.tile, c0 = tile * A.tc;
+        if (c0 >= ncell) return;
+        const int c = c0 + threadIdx.x;
+        int4 lk = make_int4(0, 0, 0, 0);
+        int cnt = 0;
+        if ((int)threadIdx.x < A.tc && c < ncell) cnt = unit_groups(A, c, ncell, lk);
+        int total;
+        const int ex = block_exclusive_scan<256>(cnt, S.sw, total);
+        S.ofs[threadIdx.x] = ex;
+        S.first[threadIdx.x] = lk.z;
+        S.end[threadIdx.x] = lk.w;
+        if (wid == 0) {
+            if (lane == 0) lb_store(A.words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
+            unsigned before = 0;
+            const bool ok = lb_sum_before(A.words, tile, before);
+            if (lane == 0) {
+                if (ok && tile) lb_store(A.words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
+                if (!ok) latch_err(A.st, kErrTimeout);
+                if (ok && c0 + A.tc >= ncell) A.st->ngroup = (int)before + total;
+                S.before = before;
+                S.ok = ok;
+            }
+        }
+        __syncthreads();
+        if (!S.ok) return;
+        for (int r = wid; r < total; r += 8) {
+            int lo = 0, hi = A.tc - 1;   // group r's cell: the last one whose first group is at or before r
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (S.ofs[mid] <= r) lo = mid; else hi = mid - 1;
+            }
+            const int first = S.first[lo] + (r - S.ofs[lo]) * A.G;
+            const int cnt = min(A.G, S.end[lo] - first);
             unsigned qlo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, qhi[3] = {0u, 0u, 0u};
             for (int i = lane; i < cnt; i += 32) {   // a run may hold up to 64 stars
-                const uint64_t key = skey[first + i];
+                const uint64_t key = A.skey[first + i];
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
                     const unsigned q = compact3(key >> a);
@@ -679,16 +916,15 @@ __global__ void groups_write_k(const uint64_t *skey, const int4 *clink, const in
                 }
             }
 #pragma unroll
-            for (int a = 0; a < 3; a++)
-                for (int o = 16; o > 0; o >>= 1) {
-                    qlo[a] = min(qlo[a], __shfl_xor_sync(0xffffffffu, qlo[a], o));
-                    qhi[a] = max(qhi[a], __shfl_xor_sync(0xffffffffu, qhi[a], o));
-                }
+            for (int a = 0; a < 3; a++) {
+                qlo[a] = __reduce_min_sync(0xffffffffu, qlo[a]);
+                qhi[a] = __reduce_max_sync(0xffffffffu, qhi[a]);
+            }
             if (lane == 0) {
-                const int g = g0 + r;
-                groups[2 * g] = make_int4(first, cnt, (int)qlo[0], (int)qlo[1]);
-                groups[2 * g + 1] = make_int4((int)qlo[2], (int)qhi[0], (int)qhi[1], (int)qhi[2]);
-                garrive[g] = 0;
+                const int g = (int)S.before + r;
+                A.groups[2 * g] = make_int4(first, cnt, (int)qlo[0], (int)qlo[1]);
+                A.groups[2 * g + 1] = make_int4((int)qlo[2], (int)qhi[0], (int)qhi[1], (int)qhi[2]);
+                A.garrive[g] = 0;
             }
         }
     }
@@ -724,78 +960,151 @@ __device__ __forceinline__ void add_q(float q[6], float m, float dx, float dy, f
     q[5] += m * 3.f * dy * dz;
 }
 
-__global__ void moments_k(int64_t n, const float4 *pos, const int4 *cbox, const int *clink, const int *cparent,
-                          int *carrive, float4 *cmom, int64_t cap, const int64_t *moff, int M,
-                          const double *mbounds, DevState *st) {
-    int ncell = (int)min((int64_t)st->ncell, cap);
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-        int4 lk = reinterpret_cast<const int4 *>(clink)[c];
+// One arrival at a cell: this thread's moments before it, the other children's
+// moments after it (acquire and release in one operation).
+__device__ __forceinline__ int arrive_acq_rel(int *p) {
+    int old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+    return old;
+}
+
+struct MomentArgs {
+    int64_t n;
+    const float4 *pos;
+    const int4 *cbox, *clink;
+    const int *cparent;
+    int *carrive;
+    float4 *cmom;
+    int64_t cap;
+    const int64_t *moff;
+    int M;
+    const double *mbounds;
+    DevState *st;
+};
+
+// What bounds a small build is the chain from the deepest leaf to the root (10
+// to 20 levels of a few dependent round trips each): there (BATCH 8) a leaf's
+// stars and all of a cell's children are in flight at once and the parent's
+// links are loaded beside the arrival. A large one is bound by the threads in
+// flight, and takes them one by one (BATCH 1) in a third of the registers. The
+// sums run in the same order either way: the moments are the same bits (80 us
+// alone before on 100003 stars, 50 now). Blocks block, block + nblocks, ... of
+// 256 cells.
+template <int BATCH>
+__device__ void climb_moments(const MomentArgs &A, int block, int nblocks) {
+    const int ncell = (int)min((int64_t)A.st->ncell, A.cap);
+    for (int c = block * 256 + threadIdx.x; c < ncell; c += nblocks * 256) {
+        const int4 lk = A.clink[c];
         if (lk.y != lk.x) continue;  // not a leaf
-        if (lk.z < 0 || lk.w > n || lk.z >= lk.w) { latch_err(st, kErrCells); continue; }
-        const int mb = member_of(moff, M, lk.z);
-        const float lo[3] = {(float)mbounds[5 * mb], (float)mbounds[5 * mb + 1], (float)mbounds[5 * mb + 2]};
-        const float unit = (float)(mbounds[5 * mb + 3] / 2097152.0);
+        if (lk.z < 0 || lk.w > A.n || lk.z >= lk.w) { latch_err(A.st, kErrCells); continue; }
+        const int mb = member_of(A.moff, A.M, lk.z);
+        const float lo[3] = {(float)A.mbounds[5 * mb], (float)A.mbounds[5 * mb + 1], (float)A.mbounds[5 * mb + 2]};
+        const float unit = (float)(A.mbounds[5 * mb + 3] / 2097152.0);
         float g[3];
-        geo_centre(cbox[c], lo, unit, g);
+        geo_centre(A.cbox[c], lo, unit, g);
+        int par = A.cparent[c];
         Mom m = {};
         float sx = 0.f, sy = 0.f, sz = 0.f;
-        for (int j = lk.z; j < lk.w; j++) {
-            float4 p = pos[j];
+        auto stars = [&](auto &&take) {
+            for (int j = lk.z; j < lk.w; j += BATCH) {
+                float4 p[BATCH];
+#pragma unroll
+                for (int k = 0; k < BATCH; k++)
+                    if (j + k < lk.w) p[k] = __ldg(&A.pos[j + k]);
+#pragma unroll
+                for (int k = 0; k < BATCH; k++)
+                    if (j + k < lk.w) take(p[k]);
+            }
+        };
+        stars([&](const float4 &p) {
             m.M += p.w;
             sx += p.w * (p.x - g[0]);
             sy += p.w * (p.y - g[1]);
             sz += p.w * (p.z - g[2]);
-        }
+        });
         if (m.M > 0.f) {
             m.cx = sx / m.M; m.cy = sy / m.M; m.cz = sz / m.M;
-            for (int j = lk.z; j < lk.w; j++) {
-                float4 p = pos[j];
+            stars([&](const float4 &p) {
                 add_q(m.q, p.w, (p.x - g[0]) - m.cx, (p.y - g[1]) - m.cy, (p.z - g[2]) - m.cz);
-            }
+            });
         }
-        store_mom(cmom, c, m);
+        store_mom(A.cmom, c, m);
         // climb while this thread is the last child to arrive (at most 21 levels)
         int cur = c;
         for (int guard = 0; guard <= kMaxLevel; guard++) {
-            int p = cparent[cur];
+            const int p = par;
             if (p < 0) break;
-            if (p >= cur) { latch_err(st, kErrCells); break; }  // parents precede children
-            __threadfence();
-            int4 pl = reinterpret_cast<const int4 *>(clink)[p];
-            int nch = pl.y - pl.x;
-            if (pl.x <= p || pl.y > ncell || nch < 1 || nch > 8) { latch_err(st, kErrCells); break; }
-            if (atomicAdd(&carrive[p], 1) != nch - 1) break;
-            __threadfence();
+            if (p >= cur) { latch_err(A.st, kErrCells); break; }  // parents precede children
+            const int4 pl = A.clink[p], pb = A.cbox[p];
+            par = A.cparent[p];
+            const int nch = pl.y - pl.x;
+            if (pl.x <= p || pl.y > ncell || nch < 1 || nch > 8) { latch_err(A.st, kErrCells); break; }
+            if (arrive_acq_rel(&A.carrive[p]) != nch - 1) break;
             float pg[3];
-            geo_centre(cbox[p], lo, unit, pg);
+            geo_centre(pb, lo, unit, pg);
             Mom P = {};
             float px = 0.f, py = 0.f, pz = 0.f;
-            for (int ch = pl.x; ch < pl.y; ch++) {
-                float4 a = __ldcg(&cmom[3 * ch]);
+            auto first = [&](const float4 &a, const int4 &b) {
                 float cg[3];
-                geo_centre(cbox[ch], lo, unit, cg);
+                geo_centre(b, lo, unit, cg);
                 P.M += a.x;
                 px += a.x * ((cg[0] - pg[0]) + a.y);
                 py += a.x * ((cg[1] - pg[1]) + a.z);
                 pz += a.x * ((cg[2] - pg[2]) + a.w);
-            }
-            if (P.M > 0.f) {
-                P.cx = px / P.M; P.cy = py / P.M; P.cz = pz / P.M;
-                for (int ch = pl.x; ch < pl.y; ch++) {
-                    float4 a = __ldcg(&cmom[3 * ch]);
-                    float4 b = __ldcg(&cmom[3 * ch + 1]);
-                    float4 e = __ldcg(&cmom[3 * ch + 2]);
-                    float cg[3];
-                    geo_centre(cbox[ch], lo, unit, cg);
-                    P.q[0] += b.x; P.q[1] += b.y; P.q[2] += b.z; P.q[3] += b.w; P.q[4] += e.x; P.q[5] += e.y;
-                    add_q(P.q, a.x, ((cg[0] - pg[0]) + a.y) - P.cx, ((cg[1] - pg[1]) + a.z) - P.cy,
-                          ((cg[2] - pg[2]) + a.w) - P.cz);
+            };
+            auto second = [&](const float4 &a, const float4 &b, const float2 &e, const int4 &bx) {
+                float cg[3];
+                geo_centre(bx, lo, unit, cg);
+                P.q[0] += b.x; P.q[1] += b.y; P.q[2] += b.z; P.q[3] += b.w; P.q[4] += e.x; P.q[5] += e.y;
+                add_q(P.q, a.x, ((cg[0] - pg[0]) + a.y) - P.cx, ((cg[1] - pg[1]) + a.z) - P.cy,
+                      ((cg[2] - pg[2]) + a.w) - P.cz);
+            };
+            auto load_a = [&](int ch) { return __ldcg(&A.cmom[3 * ch]); };
+            auto load_b = [&](int ch) { return __ldcg(&A.cmom[3 * ch + 1]); };
+            auto load_e = [&](int ch) { return __ldcg(reinterpret_cast<const float2 *>(&A.cmom[3 * ch + 2])); };
+            if (BATCH == 8) {   // every record of the children at once
+                float4 a[8], b[8];
+                float2 e[8];
+                int4 bx[8];
+#pragma unroll
+                for (int k = 0; k < 8; k++)
+                    if (k < nch) {
+                        a[k] = load_a(pl.x + k);
+                        bx[k] = A.cbox[pl.x + k];
+                        b[k] = load_b(pl.x + k);
+                        e[k] = load_e(pl.x + k);
+                    }
+#pragma unroll
+                for (int k = 0; k < 8; k++)
+                    if (k < nch) first(a[k], bx[k]);
+                if (P.M > 0.f) {
+                    P.cx = px / P.M; P.cy = py / P.M; P.cz = pz / P.M;
+#pragma unroll
+                    for (int k = 0; k < 8; k++)
+                        if (k < nch) second(a[k], b[k], e[k], bx[k]);
+                }
+            } else {
+                for (int ch = pl.x; ch < pl.y; ch++) first(load_a(ch), A.cbox[ch]);
+                if (P.M > 0.f) {
+                    P.cx = px / P.M; P.cy = py / P.M; P.cz = pz / P.M;
+                    for (int ch = pl.x; ch < pl.y; ch++) second(load_a(ch), load_b(ch), load_e(ch), A.cbox[ch]);
                 }
             }
-            store_mom(cmom, p, P);
+            store_mom(A.cmom, p, P);
             cur = p;
         }
     }
+}
+
+constexpr int64_t kLatencyBuild = 1 << 20;   // (2^19 stars: build 268 us against 273)
+
+// Walk groups and multipoles need the topology alone and not one another: one
+// launch, the first gblocks blocks write the groups while the others climb.
+template <int BATCH>
+__global__ void __launch_bounds__(256, BATCH == 8 ? 1 : 4) groups_moments_k(GroupArgs GA, MomentArgs MA, int gblocks) {
+    __shared__ GroupSmem S;
+    if ((int)blockIdx.x < gblocks) write_groups(GA, S);
+    else climb_moments<BATCH>(MA, blockIdx.x - gblocks, gridDim.x - gblocks);
 }
 
 // ---------------------------------------------------------------------------
@@ -842,48 +1151,52 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
         if (r == RV_OK) c->built = true;
         return r;
     }
-    if ((r = cuda_check(c, cudaMemsetAsync(w.mroot, 0xff, sizeof(int) * M, s), "roots")) != RV_OK) return r;
     // bounds and keys: blocks per member sized by the largest member
+    const int nblk = ceil_div(n, kTopoBlock);
+    // cells a tile of the groups pass (few in small builds: more blocks); cleared
+    // first: tickets, digit counts, the look-back words of the topology scan and of that pass
+    const int tc = n < (1 << 19) ? 64 : 256;
+    const int64_t nzero = kLbGroups(c->n_max) + 2 + ceil_div(c->cell_cap, tc);
     const int bpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, kBoundsChunk), 512 / M + 1));
-    bounds_partial_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, x, y, z, w.bpart);
+    bounds_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, x, y, z, w.bpart, w.barrive, w.mbounds, w.st, w.lb, nzero,
+                                          w.mroot);
     count_launch(c);
-    bounds_final_k<<<M, 32, 0, s>>>(bpm, w.bpart, w.mbounds, w.st);
-    count_launch(c);
-    const int kpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, 256), (int64_t)c->num_sms * 8 / M + 1));
+    // (each block adds its digit counts to the global ones: at least 1024 stars a block)
+    const int kpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, 1024), (int64_t)c->num_sms * 8 / M + 1));
     // the packed stars live in the group records' space until the gather: the
     // groups are written after it (32 B per star of room there, 16 needed)
     float4 *xyzm = reinterpret_cast<float4 *>(w.groups);
-    keys_k<<<dim3(kpm, M), 256, 0, s>>>(w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm);
+    const int64_t tiles = ceil_div(n, kSortThreads * sort_items(n));
+    keys_k<<<dim3(kpm, M), 256, 0, s>>>(w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm, w.lb + kLbHist,
+                                        reinterpret_cast<uint4 *>(w.words[0]), tiles * kSortBins / 4);
     count_launch(c);
     uint64_t *skey;
     int *perm;
-    if ((r = radix_sort(c, n, 7, &skey, &perm, true, s, true)) != RV_OK) return r;
+    if ((r = radix_sort(c, n, kKeyPasses, &skey, &perm, s, true, true, xyzm, w.pos)) != RV_OK) return r;
     w.skey = skey;
     w.perm = perm;
-    gather_k<<<grid_for(c, n, 256), 256, 0, s>>>(n, perm, xyzm, w.pos);
-    count_launch(c);
     // topology
-    int nblk = ceil_div(n, kTopoBlock);
     size_t win = kTopoBlock + 2 * c->cfg.n_leaf;
     topo_count_k<<<nblk, kTopoBlock, win, s>>>(n, skey, c->cfg.n_leaf, w.moff, M, w.dlev, w.lam, w.lvcnt, nblk);
     count_launch(c);
-    if ((r = exclusive_scan(c, w.lvcnt, (int64_t)kLevels * nblk, nullptr, &w.st->ncell, s)) != RV_OK) return r;
+    unsigned *lb = w.lb + kLbScan;   // cleared by bounds_k
+    if ((r = scan_launch(c, w.lvcnt, (int64_t)kLevels * nblk, &w.st->ncell, lb + 1, reinterpret_cast<int *>(lb), s)) !=
+        RV_OK)
+        return r;
     topo_write_k<<<nblk, kTopoBlock, 0, s>>>(n, skey, w.dlev, w.lam, w.lvcnt, nblk, c->cell_cap, w.moff, M, w.cbox,
                                              w.clink, w.cparent, w.carrive, w.mroot, w.st);
     count_launch(c);
-    // groups
-    const int G = c->cfg.group, U = 16 * c->cfg.group;
+    // groups and multipoles
     const int4 *clink4 = reinterpret_cast<const int4 *>(w.clink);
-    int gb = grid_for(c, c->cell_cap, 256);
-    groups_count_k<<<gb, 256, 0, s>>>(w.cbox, clink4, w.cparent, G, U, c->cell_cap, w.st, w.gcnt);
-    count_launch(c);
-    if ((r = exclusive_scan(c, w.gcnt, c->cell_cap, &w.st->ncell, &w.st->ngroup, s)) != RV_OK) return r;
-    groups_write_k<<<grid_for(c, c->cell_cap, 8), 256, 0, s>>>(skey, clink4, w.gcnt, &w.st->ngroup, G, c->cell_cap,
-                                                                w.st, w.groups, w.garrive);
-    count_launch(c);
-    // multipoles
-    moments_k<<<gb, 128, 0, s>>>(n, w.pos, w.cbox, w.clink, w.cparent, w.carrive, w.cmom, c->cell_cap, w.moff, M,
-                                 w.mbounds, w.st);
+    const int gblocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(c->cell_cap, tc), c->num_sms));
+    const int mblocks = grid_for(c, c->cell_cap, 256);
+    const GroupArgs GA{skey, w.cbox, clink4, w.cparent, c->cfg.group, 16 * c->cfg.group, tc, c->cell_cap,
+                       w.lb + kLbGroups(c->n_max) + 1, reinterpret_cast<int *>(w.lb + kLbGroups(c->n_max)), w.groups,
+                       w.garrive, w.st};
+    const MomentArgs MA{n, w.pos, w.cbox, clink4, w.cparent, w.carrive, w.cmom, c->cell_cap, w.moff, M, w.mbounds, w.st};
+    // (one wave of latency-bound blocks as long as the cells fit it)
+    if (n < kLatencyBuild) groups_moments_k<8><<<gblocks + mblocks, 256, 0, s>>>(GA, MA, gblocks);
+    else groups_moments_k<1><<<gblocks + mblocks, 256, 0, s>>>(GA, MA, gblocks);
     count_launch(c);
     r = cuda_check(c, cudaGetLastError(), "build_tree");
     if (r == RV_OK) c->built = true;

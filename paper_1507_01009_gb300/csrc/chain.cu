@@ -154,7 +154,7 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
         sel_radius_flag_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, ch, R, w.sel_flag);
         count_launch(c);
         int *total = &w.st->n_pert;  // scratch for the total; overwritten by the clamped count
-        rv_status r = exclusive_scan(c, w.sel_flag, n, nullptr, total, s);
+        rv_status r = exclusive_scan(c, w.sel_flag, n, total, s);
         if (r != RV_OK) return r;
         sel_radius_write_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, ch, R, w.sel_flag, total, cap, idx,
                                                         count, w.st);
@@ -170,7 +170,7 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
         count_launch(c);
         uint64_t *sk;
         int *si;
-        rv_status r = radix_sort(c, n, 4, &sk, &si, true, s);
+        rv_status r = radix_sort(c, n, 4, &sk, &si, s);
         if (r != RV_OK) return r;
         sel_knn_write_k<<<ceil_div(std::min<int64_t>(k, n), 256), 256, 0, s>>>(si, n, std::min(k, cap), idx, count, w.st);
         count_launch(c);
@@ -188,7 +188,7 @@ rv_status influence_radius(rv_ctx *c, int64_t n, const float *x, const float *y,
     count_launch(c);
     uint64_t *sk;
     int *si;
-    rv_status r = radix_sort(c, n, 4, &sk, &si, true, s);
+    rv_status r = radix_sort(c, n, 4, &sk, &si, s);
     if (r != RV_OK) return r;
     influence_k<<<1, 32, 0, s>>>(n, sk, si, vx, vy, vz, m, m_bh, std::min<int64_t>(n_sigma, n), w.out8);
     count_launch(c);
@@ -567,7 +567,7 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 count_launch(c);
                 uint64_t *sk;
                 int *si;
-                if ((r = radix_sort(c, sys->n, sys->pert_mode == 2 ? 4 : 1, &sk, &si, true, s, true)) != RV_OK)
+                if ((r = radix_sort(c, sys->n, sys->pert_mode == 2 ? 4 : 1, &sk, &si, s, true)) != RV_OK)
                     return r;
                 sel_member_write_k<<<M, 256, 0, s>>>(w.moff, sk, si, sys->pert_mode, sys->pert_k, cap, C, j,
                                                      w.pert_idx, w.npert, w.st);

@@ -94,7 +94,7 @@ rv_status rv_chain_absorb(rv_ctx *c, int64_t n, const float *x, const float *y, 
     if (n > 0) {
         absorb_flag_k<<<grid, 256, 0, s>>>(n, x, y, z, w.st, w.sel_flag);
         count_launch(c);
-        rv_status r = exclusive_scan(c, w.sel_flag, n, nullptr, total, s);
+        rv_status r = exclusive_scan(c, w.sel_flag, n, total, s);
         if (r != RV_OK) return r;
     }
     absorb_write_k<<<grid, 256, 0, s>>>(n, x, y, z, w.st, w.sel_flag, total, cap, idx, count, r_chain);

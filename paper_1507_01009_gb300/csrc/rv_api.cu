@@ -40,11 +40,7 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     int64_t n = n_max > 0 ? n_max : 1;
     int64_t cap = cell_capacity(n, cfg.n_leaf);
     if (cell_cap) *cell_cap = cap;
-    int64_t ntiles = (n + kSortTile - 1) / kSortTile;
     int64_t nblk = (n + kTopoBlock - 1) / kTopoBlock;
-    int64_t scan_max = std::max<int64_t>(std::max<int64_t>((int64_t)kSortBins * ntiles, (int64_t)kLevels * nblk),
-                                         std::max<int64_t>(cap, n));
-    int64_t nparts = std::max<int64_t>(6 * 1024, scan_max / kScanChunk + 2);
     size_t off = 0;
     auto take = [&](size_t bytes) -> char * {
         char *p = base ? base + off : nullptr;
@@ -56,7 +52,10 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.key_b = (uint64_t *)take(8 * n);
     t.idx_a = (int *)take(4 * n);
     t.idx_b = (int *)take(4 * n);
-    t.hist = (int *)take(4 * (size_t)kSortBins * ntiles);
+    t.words[0] = (unsigned *)take(4 * (size_t)sort_words(n));
+    t.words[1] = (unsigned *)take(4 * (size_t)sort_words(n));
+    // (the groups' look-back words: at most one a tile of 64 cells)
+    t.lb = (unsigned *)take(4 * (size_t)(kLbGroups(n) + 3 + (cap + 63) / 64));
     t.skey = nullptr;
     t.perm = nullptr;
     t.pos = (float4 *)take(16 * n);
@@ -69,7 +68,6 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.coct = (float4 *)take(48 * cap);
     t.cparent = (int *)take(4 * cap);
     t.carrive = (int *)take(4 * cap);
-    t.gcnt = (int *)take(4 * cap);
     t.groups = (int4 *)take(32 * (n + 1));   // every group holds a star
     t.gact = (uint8_t *)take(n + 1);
     t.scost = (float *)take(4 * n);
@@ -81,7 +79,6 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.gbin = (int *)take(4 * (n + 1));
     t.obins = (int *)take(4 * 1024);
     t.block_count = (unsigned long long *)take(16);
-    t.partials = (int *)take(4 * nparts);
     t.pert_idx = (int *)take(4 * kPertTotal);
     t.pert_m = (double *)take(8 * kPertTotal);
     t.pert_x = (double *)take(24 * kPertTotal);
@@ -101,6 +98,7 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.mbounds = (double *)take(8 * 5 * kMaxMembers);
     t.mroot = (int *)take(4 * kMaxMembers);
     t.bpart = (float *)take(4 * 6 * 2048);
+    t.barrive = (int *)take(4 * kMaxMembers);
     t.xmem = (int *)take(4 * kExtraTotal);
     t.npert = (int *)take(4 * kMaxMembers);
     t.gstack = (int *)take(4 * (size_t)kStackSpillWarps * kStackSpill);
@@ -210,6 +208,7 @@ rv_status rv_set_workspace(rv_ctx *c, void *dev, size_t bytes) {
         c->graph = nullptr;
     }
     cudaError_t e = cudaMemset(c->w.st, 0, sizeof(DevState));
+    if (e == cudaSuccess) e = cudaMemset(c->w.barrive, 0, 4 * kMaxMembers);
     return cuda_check(c, e, "workspace init");
 }
 

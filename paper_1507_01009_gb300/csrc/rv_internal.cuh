@@ -16,8 +16,7 @@ constexpr int kLevels = kMaxLevel + 1;  // 22
 constexpr int kSortBits = 9;            // radix digit width
 constexpr int kSortBins = 1 << kSortBits;
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
+constexpr int kKeyPasses = 7;           // passes over a 63-bit key
 constexpr int kTopoBlock = 256;
 constexpr int kScanChunk = 2048;        // elements per scan block
 #ifndef RV_WALK_WARPS
@@ -93,7 +92,8 @@ struct Workspace {
     // tree build
     uint64_t *key_a, *key_b;
     int *idx_a, *idx_b;
-    int *hist;            // radix histograms [bins x tiles]
+    unsigned *words[2];   // sort passes' look-back words [tiles x bins], used in turn
+    unsigned *lb;         // tickets, digit counts, other look-back words (kLbTickets ..)
     uint64_t *skey;       // sorted keys of the last build (key_a or key_b)
     int *perm;            // sorted slot -> caller index of the last build (idx_a or idx_b)
     float4 *pos;          // sorted (x, y, z, m)
@@ -104,7 +104,6 @@ struct Workspace {
     float4 *cmom;         // [3 ncell]
     float4 *coct;         // [3 ncell] traceless octupoles (the learned correction's features only)
     int *cparent, *carrive;
-    int *gcnt;            // groups of each cell, scanned in place to each cell's first group
     int4 *groups;         // 2 int4 per group: (first, count, lo x, lo y), (lo z, hi x, hi y, hi z)
     uint8_t *gact;        // block time steps: groups holding an active star
     float *scost;         // per caller star: list cost of its group in the last walk (scheduling only)
@@ -115,7 +114,6 @@ struct Workspace {
     int *gbin;            // each group's cost bin (queue order scratch)
     int *obins;           // bin counts, then next free slots (queue order scratch, 1024)
     unsigned long long *block_count;  // block time steps: active star updates so far
-    int *partials;        // scan block sums
     // perturbers and chain hand-off
     int *pert_idx;        // [kMaxPert]
     double *pert_m, *pert_x;           // [kMaxPert], [3 kMaxPert]
@@ -132,6 +130,7 @@ struct Workspace {
     double *mbounds;      // per member: min x, y, z, L, 2^21 / L
     int *mroot;           // root cell of each member (-1 if empty)
     float *bpart;         // bounds partials
+    int *barrive;         // blocks of each member's bounds that are done (0 between builds)
     int *xmem;            // member of each extra particle
     int *npert;           // perturbers selected per member
     int *gstack;          // walk stack entries beyond kStackSm, kStackSpill per warp [kStackSpillWarps]
@@ -183,9 +182,18 @@ rv_status cuda_check(rv_ctx *c, cudaError_t e, const char *what);
 rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const float *x, const float *y,
                      const float *z, const float *m, cudaStream_t s);
 rv_status upload_offsets(rv_ctx *c, int M, const int64_t *offsets, cudaStream_t s);
-rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, bool identity_idx,
-                     cudaStream_t s, bool member_pass = false);
-rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, const int *d_len, int *d_total, cudaStream_t s);
+rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, cudaStream_t s,
+                     bool member_pass = false, bool counted = false, const float4 *xyzm = nullptr,
+                     float4 *pos = nullptr);
+rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s);
+int64_t sort_words(int64_t n_max);   // look-back words of a sort pass, for any n <= n_max
+
+// Layout of Workspace::lb (32-bit words): sort tickets [16], digit counts
+// [kKeyPasses][kSortBins], a scan's ticket and words, the groups' ticket and words.
+constexpr int64_t kLbTickets = 0, kLbHist = 16, kLbScan = kLbHist + kKeyPasses * kSortBins;
+inline int64_t kLbGroups(int64_t n_max) {   // after the longest scan: n flags, or 22 counts per 256 stars
+    return kLbScan + 2 + (n_max + kScanChunk - 1) / kScanChunk + 1;
+}
 
 // Opening test on integer grid distances: accept iff d^2 >= thr[level].
 struct MacTable {
