@@ -102,6 +102,219 @@ __global__ void sel_knn_write_k(const int *sorted_idx, int64_t n, int k, int *id
     }
 }
 
+// ---------------------------------------------------------------------------
+// k nearest by selection: the stars in order of (FP32 squared distance bits,
+// caller index), the first k of them, without sorting the rest. (1) counts of the
+// distances' leading 11 bits (exponent and three mantissa bits: an eighth of
+// an octave a bin); (2) the stars up to the bin that holds the k-th are gathered,
+// in any order -- about 1.1 to 1.2 k of them unless many stars lie at nearly
+// one distance; (3) one block a member sorts them. If they do not fit its shared
+// memory it first narrows them digit by digit of the 64-bit (distance, index)
+// value, which is different for every star, so this ends for any input.
+// Two reads of the positions instead of a four-pass radix sort of all stars:
+// 256 of 2^20 stars 111 -> 30 us of kernels (cold). Members side by side (grid y): a member's
+// candidates go to its own slots of the buffer.
+// ---------------------------------------------------------------------------
+constexpr int kSelCap = 8192;        // candidates a block sorts in shared memory
+constexpr int kSelMaxK = kMaxPert;   // larger selections sort everything
+
+struct SelNear {
+    const int64_t *moff;      // member offsets (nullptr: one member of n stars)
+    int64_t n;
+    const float *x, *y, *z;
+    const float *cdev;        // centres (x, y, z, .), member m's at 4 (m C + j); nullptr: chost
+    int C, j;
+    float3 chost;
+    int k, cap;               // wanted; slots of a member's output
+    int *hist, *ncand;        // [members][kSelBins], [members]: zero before and after
+    uint64_t *cand, *alt;     // [n] each
+    int *idx, *count;         // chain ch's output at idx + ch cap, count + ch (ch = m C + j)
+    DevState *st;
+    bool report;              // one member: st->n_pert as well
+};
+
+__device__ __forceinline__ int near_bin(unsigned key) { return (int)min(key >> 20, (unsigned)kSelBins - 1); }
+
+__device__ __forceinline__ float3 near_centre(const SelNear &A, int m) {
+    const float *q = A.cdev ? A.cdev + 4 * ((int64_t)m * A.C + A.j) : nullptr;
+    return q ? make_float3(q[0], q[1], q[2]) : A.chost;
+}
+
+// Calls take(key, i) for the block's stars, four of a thread's loaded at once.
+template <typename F>
+__device__ __forceinline__ void near_scan(const SelNear &A, const float3 &c, int64_t s, int64_t e, F &&take) {
+    const int64_t stride = (int64_t)gridDim.x * 256;
+    for (int64_t i = s + (int64_t)blockIdx.x * 256 + threadIdx.x; i < e; i += 4 * stride) {
+        unsigned key[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int64_t q = i + u * stride;
+            if (q < e) key[u] = __float_as_uint(dist2_f32(A.x[q], A.y[q], A.z[q], c.x, c.y, c.z));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i + u * stride < e) take(key[u], i + u * stride);
+    }
+}
+
+__global__ void __launch_bounds__(256) near_hist_k(SelNear A) {
+    __shared__ int h[kSelBins];
+    const int m = blockIdx.y;
+    for (int b = threadIdx.x; b < kSelBins; b += 256) h[b] = 0;
+    const int64_t s = A.moff ? A.moff[m] : 0, e = A.moff ? A.moff[m + 1] : A.n;
+    const float3 c = near_centre(A, m);
+    __syncthreads();
+    near_scan(A, c, s, e, [&](unsigned key, int64_t) { atomicAdd(&h[near_bin(key)], 1); });
+    __syncthreads();
+    for (int b = threadIdx.x; b < kSelBins; b += 256)
+        if (h[b]) atomicAdd(&A.hist[(int64_t)m * kSelBins + b], h[b]);
+}
+
+// Inclusive sum over the block of one value a thread (NT threads).
+template <int NT>
+__device__ __forceinline__ int block_inclusive_sum(int v, int *sw) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) sw[wid] = x;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < wid; w++) before += sw[w];
+    return before + x;
+}
+
+// The first bin at which the running count of h reaches `need` (need >= 1, not
+// above the total), and the count before it; the same in every thread.
+template <int NT>
+__device__ __forceinline__ void find_bin(const int *h, int need, int *sw, int *found, int &bin, int &before) {
+    constexpr int PER = kSelBins / NT;
+    int v[PER], s = 0;
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+        v[q] = h[threadIdx.x * PER + q];
+        s += v[q];
+    }
+    const int incl = block_inclusive_sum<NT>(s, sw);
+    int run = incl - s;
+    if (run < need && incl >= need) {
+#pragma unroll
+        for (int q = 0; q < PER; q++) {
+            if (run < need && run + v[q] >= need) {
+                found[0] = threadIdx.x * PER + q;
+                found[1] = run;
+            }
+            run += v[q];
+        }
+    }
+    __syncthreads();
+    bin = found[0];
+    before = found[1];
+}
+
+__global__ void __launch_bounds__(256) near_gather_k(SelNear A) {
+    __shared__ int sw[8], found[2];
+    const int m = blockIdx.y;
+    const int64_t s = A.moff ? A.moff[m] : 0, e = A.moff ? A.moff[m + 1] : A.n;
+    const int need = (int)min((int64_t)A.k, e - s);
+    if (need <= 0) return;
+    int bin, before;
+    find_bin<256>(A.hist + (int64_t)m * kSelBins, need, sw, found, bin, before);
+    const float3 c = near_centre(A, m);
+    near_scan(A, c, s, e, [&](unsigned key, int64_t i) {
+        if (near_bin(key) <= bin) {
+            const unsigned act = __activemask();
+            const int leader = __ffs(act) - 1;
+            int at = 0;
+            if ((int)(threadIdx.x & 31) == leader) at = atomicAdd(&A.ncand[m], __popc(act));
+            at = __shfl_sync(act, at, leader) + __popc(act & lanemask_lt());
+            A.cand[s + at] = ((uint64_t)key << 32) | (unsigned)i;
+        }
+    });
+}
+
+__global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
+    extern __shared__ __align__(16) char near_smem[];
+    uint64_t *v = reinterpret_cast<uint64_t *>(near_smem);   // [kSelCap]
+    __shared__ int h[kSelBins], sw[32], found[2], nacc, nrem;
+    const int m = blockIdx.x, t = threadIdx.x;
+    const int64_t s = A.moff ? A.moff[m] : 0, e = A.moff ? A.moff[m + 1] : A.n;
+    const int64_t ch = (int64_t)m * A.C + A.j;
+    int *hist = A.hist + (int64_t)m * kSelBins;
+    const int take = (int)min((int64_t)A.k, e - s);
+    int rem = take > 0 ? A.ncand[m] : 0, acc = 0;
+    __syncthreads();
+    for (int b = t; b < kSelBins; b += 1024) hist[b] = 0;   // ready for the next selection
+    if (t == 0) {
+        A.ncand[m] = 0;
+        nacc = 0;
+    }
+    uint64_t *a = A.cand + s, *o = A.alt + s;
+    for (int shift = 53; acc + rem > kSelCap; shift = max(shift - 11, 0)) {
+        for (int b = t; b < kSelBins; b += 1024) h[b] = 0;
+        if (t == 0) nrem = 0;
+        __syncthreads();
+        for (int i = t; i < rem; i += 1024) atomicAdd(&h[(int)(a[i] >> shift) & (kSelBins - 1)], 1);
+        __syncthreads();
+        int bin, before;
+        find_bin<1024>(h, take - acc, sw, found, bin, before);
+        for (int i = t; i < rem; i += 1024) {
+            const uint64_t w = a[i];
+            const int d = (int)(w >> shift) & (kSelBins - 1);
+            if (d < bin) v[atomicAdd(&nacc, 1)] = w;          // among the k nearest: at most take of these
+            else if (d == bin) o[atomicAdd(&nrem, 1)] = w;
+        }
+        __syncthreads();
+        acc = nacc;
+        rem = nrem;
+        uint64_t *q = a;
+        a = o;
+        o = q;
+        __syncthreads();
+    }
+    for (int i = t; i < rem; i += 1024) v[acc + i] = a[i];
+    int size = 2;
+    while (size < acc + rem) size <<= 1;
+    for (int i = acc + rem + t; i < size; i += 1024) v[i] = ~0ull;
+    for (int k = 2; k <= size; k <<= 1)   // bitonic sort
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            for (int q = t; q < size / 2; q += 1024) {
+                const int i = 2 * q - (q & (j - 1));   // the pair's lower place
+                const uint64_t lo = v[i], hi = v[i + j];
+                if ((lo > hi) == ((i & k) == 0)) {
+                    v[i] = hi;
+                    v[i + j] = lo;
+                }
+            }
+        }
+    __syncthreads();
+    const int kk = min(take, A.cap);
+    for (int i = t; i < kk; i += 1024) A.idx[ch * A.cap + i] = (int)(unsigned)v[i];
+    if (t == 0) {
+        A.count[ch] = kk;
+        if (A.report) A.st->n_pert = kk;
+        else if (take > A.cap) latch_err(A.st, kErrPert);
+    }
+}
+
+static rv_status select_nearest(rv_ctx *c, const SelNear &A, int members, int64_t largest, cudaStream_t s) {
+    const size_t smem = sizeof(uint64_t) * kSelCap;
+    cudaError_t e = cudaFuncSetAttribute(near_sort_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_check(c, e, "select nearest");
+    // about 1024 stars a block, four blocks an SM over all members
+    const int bx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(largest, 1024), (int64_t)c->num_sms * 4 / members + 1));
+    near_hist_k<<<dim3(bx, members), 256, 0, s>>>(A);
+    near_gather_k<<<dim3(bx, members), 256, 0, s>>>(A);
+    near_sort_k<<<members, 1024, smem, s>>>(A);
+    c->launches += 3;
+    return cuda_check(c, cudaGetLastError(), "select nearest");
+}
+
 // Eq. 1 ingredients from the stars sorted by FP32 squared distance (keys =
 // the d2 bits, ties by index): r(<2 M_bh), sigma of the k nearest, M_bh / sigma^2.
 // One thread, sums in distance order in FP64, exactly as the rule reads.
@@ -166,6 +379,12 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
         }
         // the sort buffers are shared with the tree build: the tree is invalid afterwards
         c->built = false;
+        if (std::min<int64_t>(k, n) <= kSelMaxK) {
+            // (one member: an output shorter than k is simply the nearest cap of them)
+            const SelNear A{nullptr, n, x, y, z, centre_dev, 1, 0, make_float3(ch.x, ch.y, ch.z), std::min(k, cap), cap,
+                            w.selhist, w.selcand, w.key_a, w.key_b, idx, count, w.st, true};
+            if (A.k > 0) return select_nearest(c, A, 1, n, s);
+        }
         sel_knn_keys_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, make_float3(ch.x, ch.y, ch.z), w.key_a);
         count_launch(c);
         uint64_t *sk;
@@ -560,6 +779,15 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 if (r != RV_OK) return r;
             } else {
                 // the sort buffers are shared with the tree build, which comes next
+                if (sys->pert_mode == 2 && sys->pert_k > 0) {
+                    const SelNear A{w.moff, sys->n, sys->x, sys->y, sys->z, w.extra_xyzm, C, j, make_float3(0.f, 0.f, 0.f),
+                                    sys->pert_k, cap, w.selhist, w.selcand, w.key_a, w.key_b, w.pert_idx, w.npert, w.st,
+                                    false};
+                    int64_t big = 1;
+                    for (int k = 0; k < M; k++) big = std::max<int64_t>(big, off[k + 1] - off[k]);
+                    if ((r = select_nearest(c, A, M, big, s)) != RV_OK) return r;
+                    continue;
+                }
                 const int bpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(c->max_member, 256), 64));
                 const SelRule R = sel_rule(sys->pert_mode, sys->pert_radius, sys->m, sys->pert_gamma);
                 sel_member_keys_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, sys->x, sys->y, sys->z, w.extra_xyzm, C,

@@ -94,6 +94,8 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.pflag = (uint8_t *)take(n);
     t.red = (double *)take(8 * 9 * kRedSlots);
     t.sel_flag = (int *)take(4 * n);
+    t.selhist = (int *)take(4 * (size_t)kMaxMembers * kSelBins);
+    t.selcand = (int *)take(4 * kMaxMembers);
     t.moff = (int64_t *)take(8 * (kMaxMembers + 1));
     t.mbounds = (double *)take(8 * 5 * kMaxMembers);
     t.mroot = (int *)take(4 * kMaxMembers);
@@ -209,6 +211,8 @@ rv_status rv_set_workspace(rv_ctx *c, void *dev, size_t bytes) {
     }
     cudaError_t e = cudaMemset(c->w.st, 0, sizeof(DevState));
     if (e == cudaSuccess) e = cudaMemset(c->w.barrive, 0, 4 * kMaxMembers);
+    if (e == cudaSuccess) e = cudaMemset(c->w.selhist, 0, 4 * (size_t)kMaxMembers * kSelBins);
+    if (e == cudaSuccess) e = cudaMemset(c->w.selcand, 0, 4 * kMaxMembers);
     return cuda_check(c, e, "workspace init");
 }
 

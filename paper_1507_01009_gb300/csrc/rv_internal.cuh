@@ -35,6 +35,7 @@ constexpr int kPertTotal = 65536;       // perturber slots over all members
 constexpr int kChainTotal = 2048;       // chain members over all members
 constexpr int kExtraTotal = kMaxMembers;  // extra particles (chain centres) over all members
 constexpr int kRedSlots = 1024;         // energy partial-sum blocks over all members
+constexpr int kSelBins = 2048;          // nearest selection: bins of the distances' leading bits
 constexpr int kMaxChain = 250;
 constexpr int kMaxPert = 5000;
 
@@ -125,6 +126,8 @@ struct Workspace {
     uint8_t *pflag;       // [n]: 1 for the stars that are perturbers of a chain (caller order)
     double *red;          // energy partial sums
     int *sel_flag;        // perturber selection flags (n)
+    int *selhist;         // nearest selection: distance counts per member [kMaxMembers][kSelBins], 0 between calls
+    int *selcand;         // ... and candidates gathered [kMaxMembers], 0 between calls
     // members (independent systems sharing one build and one walk)
     int64_t *moff;        // member star offsets [kMaxMembers + 1]
     double *mbounds;      // per member: min x, y, z, L, 2^21 / L

@@ -66,3 +66,58 @@ def test_selections_at_tile_edges(rvmod, n):
     idx, cnt = ctx.select_perturbers(x, y, z, (0.0, 0.0, 0.0), 1, radius=0.3, cap=max(1, len(inside)))
     assert int(cnt.item()) == len(inside)
     np.testing.assert_array_equal(idx[:len(inside)].cpu().numpy(), inside)
+
+
+@pytest.mark.parametrize("n,k", [(9000, 3000), (9000, 5000), (70001, 1), (70001, 4999)])
+def test_nearest_of_many_equal_distances(rvmod, n, k):
+    """Candidates that do not fit one block's shared memory: all stars at one
+    distance (ties by index), and half of them, beside distances of 0, infinity and
+    far below the bins' resolution."""
+    import torch
+    rng = np.random.default_rng(n + k)
+    for kind in range(3):
+        x = np.full(n, 2.0, dtype=np.float32)
+        if kind == 1:
+            x[rng.permutation(n)[: n // 2]] = np.float32(3.0)
+        if kind == 2:
+            x[:] = np.float32(2.0) + rng.integers(0, 3, n).astype(np.float32) * np.float32(2.0 ** -22)
+            x[rng.permutation(n)[:5]] = [0.0, np.inf, -np.inf, 1e-30, 2.0]
+        y, z = np.zeros_like(x), np.zeros_like(x)
+        d2 = (x * x + y * y) + z * z
+        ctx = rvmod.Context(n)
+        xs = [torch.from_numpy(v).cuda() for v in (x, y, z)]
+        for _ in range(2):
+            idx, cnt = ctx.select_perturbers(*xs, (0.0, 0.0, 0.0), 2, k=k)
+            assert int(cnt.item()) == k
+            np.testing.assert_array_equal(idx[:k].cpu().numpy(), np.argsort(d2, kind="stable")[:k])
+
+
+def test_nearest_per_member(rvmod):
+    """Perturbers of every member of an ensemble (empty, smaller than k, large), by the forces they make: the
+    selection of each member equals the one of its stars alone."""
+    import torch
+    sizes, k = [40, 0, 5000, 1, 70001], 64
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    p32, m32 = hernquist32(int(off[-1]), 5)
+    M = len(sizes)
+    cm = np.full(2 * M, 0.005)
+    cx = np.tile(np.array([[0.0055, 0, 0], [-0.0055, 0, 0]]), (M, 1))
+    ctx = rvmod.Context(int(off[-1]), theta=0.5, eps_star=0.005)
+    S = rvmod.System(p32, np.zeros_like(p32), m32, chain_m=cm, chain_x=cx, chain_v=np.zeros_like(cx), pert_mode=2,
+                     pert_k=k, member_offsets=off)
+    ctx.system_forces(S)
+    at = torch.from_numpy(cx).cuda()
+    a, pot = ctx.chain_perturber_forces(S, 0.0, at)
+    ctx.sync_status()
+    a, pot = a.cpu().numpy().reshape(-1, 3), pot.cpu().numpy()
+    for i in range(M):
+        p = p32[:, off[i]:off[i + 1]]
+        d2 = (p[0] * p[0] + p[1] * p[1]) + p[2] * p[2]
+        near = np.argsort(d2, kind="stable")[:k]
+        q, w = p[:, near].astype(np.float64), m32[off[i]:off[i + 1]][near].astype(np.float64)
+        for b in (2 * i, 2 * i + 1):
+            d = q - cx[b][:, None]
+            r = np.sqrt((d * d).sum(0))
+            ref = (w * d / r ** 3).sum(1)
+            assert np.allclose(a[b], ref, rtol=1e-11, atol=1e-12 * max(1.0, np.abs(w / r ** 2).sum()))
+            assert np.isclose(pot[b], -(w / r).sum(), rtol=1e-12, atol=1e-14)
