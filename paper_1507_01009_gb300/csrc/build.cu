@@ -169,10 +169,23 @@ rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaS
 // ---------------------------------------------------------------------------
 // bounding cube
 // ---------------------------------------------------------------------------
+// The bounding cube of an axis-wise range: min x, y, z; L = max_a (max_a - min_a)
+// with FP64 differences; scale = 2^21 / L (0 if L = 0).
+__device__ __forceinline__ void cube_of(const float lo[3], const float hi[3], double out[5]) {
+    double L = 0.0;
+    for (int a = 0; a < 3; a++) {
+        bool empty = !(lo[a] <= hi[a]);
+        double e = empty ? 0.0 : __dsub_rn((double)hi[a], (double)lo[a]);
+        if (e > L) L = e;
+        out[a] = empty ? 0.0 : (double)lo[a];
+    }
+    out[3] = L;
+    out[4] = (L > 0.0) ? __ddiv_rn(2097152.0, L) : 0.0;
+}
+
 // Blocks (bx, m): member m's stars, strided by bpm blocks; the last block of a
-// member to finish reduces the blocks' partials: min per axis; L = max_a (max_a
-// - min_a) with FP64 differences; scale = 2^21 / L (min and max are exact, so
-// the order is free). The first kernel of a build, it also clears the words the
+// member to finish reduces the blocks' partials (min and max are exact, so the
+// order is free). The first kernel of a build, it also clears the words the
 // later ones count in (zero[nzero]) and the member roots.
 __global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, const float *x, const float *y,
                                                 const float *z, float *part, int *arrive, double *mbounds,
@@ -231,15 +244,7 @@ __global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, co
     warp_minmax();
     if (lane != 0) return;
     double out[5];
-    double L = 0.0;
-    for (int a = 0; a < 3; a++) {
-        bool empty = !(lo[a] <= hi[a]);
-        double e = empty ? 0.0 : __dsub_rn((double)hi[a], (double)lo[a]);
-        if (e > L) L = e;
-        out[a] = empty ? 0.0 : (double)lo[a];
-    }
-    out[3] = L;
-    out[4] = (L > 0.0) ? __ddiv_rn(2097152.0, L) : 0.0;
+    cube_of(lo, hi, out);
     for (int k = 0; k < 5; k++) {
         mbounds[5 * m + k] = out[k];
         if (m == 0) st->bounds[k] = out[k];
@@ -332,22 +337,28 @@ __device__ __forceinline__ uint32_t grid_coord_fast(float v, const GridAxis &g) 
     return grid_coord(v, g.lo, g.scale);
 }
 
-// Digit counts of one key per lane (ok: the lane has one) into the block's
-// [passes][kSortBins] counters. The high digits of a centrally concentrated
-// system hold few values: there the lanes of a warp with one digit add once.
-template <int PASSES>
-__device__ __forceinline__ void count_digits(uint64_t k, bool ok, int *h) {
-    const unsigned lt = lanemask_lt();
+// Lanes of the warp with this lane's digit, among those with ok (the others get
+// nothing useful): one ballot a bit (the ranking rounds with __match_any_sync: a
+// pass over 2^24 elements 260 us, 233 so).
+__device__ __forceinline__ unsigned match_digit(unsigned d, bool ok) {
+    unsigned m = __ballot_sync(0xffffffffu, ok);
 #pragma unroll
-    for (int p = 0; p < PASSES; p++) {
-        const int d = (int)(k >> (p * kSortBits)) & (kSortBins - 1);
-        if (p >= 3) {
-            const unsigned peers = __match_any_sync(0xffffffffu, ok ? d : -1);
-            if (ok && (peers & lt) == 0) atomicAdd(&h[p * kSortBins + d], __popc(peers));
-        } else if (ok) {
-            atomicAdd(&h[p * kSortBins + d], 1);
-        }
+    for (int b = 0; b < kSortBits; b++) {
+        const bool one = (d >> b) & 1u;
+        const unsigned v = __ballot_sync(0xffffffffu, one);
+        m &= one ? v : ~v;
     }
+    return m;
+}
+
+// Digit counts of one key into the block's [passes][kSortBins] counters. (The high
+// digits of a centrally concentrated system hold few values; shared-memory adds
+// of a whole warp to one counter still beat finding the lanes that agree: build of
+// 2^24 stars 3.40 ms, 3.60 with the four high digits added once per value.)
+template <int PASSES>
+__device__ __forceinline__ void count_digits(uint64_t k, int *h) {
+#pragma unroll
+    for (int p = 0; p < PASSES; p++) atomicAdd(&h[p * kSortBins + ((int)(k >> (p * kSortBits)) & (kSortBins - 1))], 1);
 }
 
 // Blocks (bx, m): member m's stars with member m's bounding cube. Each star's
@@ -370,19 +381,13 @@ __global__ void __launch_bounds__(256) keys_k(const int64_t *moff, int bpm, cons
                    gz = grid_axis(mbounds[5 * m + 2], sc);
     const int64_t s = moff[m], e = moff[m + 1];
     __syncthreads();
-    const int64_t w0 = s + (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31);   // the warp's first star
-    for (int64_t b = w0; b < e; b += (int64_t)bpm * 256) {
-        const int64_t i = b + (threadIdx.x & 31);
-        const bool ok = i < e;
-        uint64_t k = 0;
-        if (ok) {
-            const float xi = x[i], yi = y[i], zi = z[i];
-            k = spread3(grid_coord_fast(xi, gx)) | (spread3(grid_coord_fast(yi, gy)) << 1) |
-                (spread3(grid_coord_fast(zi, gz)) << 2);
-            key[i] = k;
-            xyzm[i] = make_float4(xi, yi, zi, mass[i]);
-        }
-        count_digits<kKeyPasses>(k, ok, h);
+    for (int64_t i = s + (int64_t)blockIdx.x * 256 + threadIdx.x; i < e; i += (int64_t)bpm * 256) {
+        const float xi = x[i], yi = y[i], zi = z[i];
+        const uint64_t k = spread3(grid_coord_fast(xi, gx)) | (spread3(grid_coord_fast(yi, gy)) << 1) |
+                           (spread3(grid_coord_fast(zi, gz)) << 2);
+        key[i] = k;
+        xyzm[i] = make_float4(xi, yi, zi, mass[i]);
+        count_digits<kKeyPasses>(k, h);
     }
     __syncthreads();
     for (int b = threadIdx.x; b < kKeyPasses * kSortBins; b += 256)
@@ -397,10 +402,8 @@ __global__ void __launch_bounds__(256) sort_hist_k(int64_t n, const uint64_t *ke
     __shared__ int h[4 * kSortBins];
     for (int b = threadIdx.x; b < 4 * kSortBins; b += 256) h[b] = 0;
     __syncthreads();
-    for (int64_t b = (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31); b < n; b += (int64_t)gridDim.x * 256) {
-        const int64_t i = b + (threadIdx.x & 31);
-        count_digits<4>(i < n ? key[i] : 0ull, i < n, h);
-    }
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
+        count_digits<4>(key[i], h);
     __syncthreads();
     for (int b = threadIdx.x; b < passes * kSortBins; b += 256)
         if (h[b]) atomicAdd(&ghist[b], (unsigned)h[b]);
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(256) sort_hist_k(int64_t n, const uint64_t *ke
 // count, a three-kernel scan and a move: seven passes 190 -> 73 us on 100003
 // stars, where launches and latency count. Large sorts are bound by the ranking
 // rounds and the short output runs (512 digits a tile of 4096: 8 elements a run;
-// 2^24 elements 260 us a pass, 1.5 TB/s).
+// 2^24 elements 233 us a pass, 1.7 TB/s).
 template <int ITEMS>
 struct SortSmem {
     unsigned short cnt[kSortThreads / 32][kSortBins];
@@ -479,7 +482,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uin
         int d = kSortBins;
         if (j < n) d = moff ? member_of(moff, M, (int64_t)ix[r]) : (int)((kk[r] >> shift) & (kSortBins - 1));
         digit[r] = d;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
+        const unsigned peers = match_digit(d, d < kSortBins);
         int before = (d < kSortBins) ? S.cnt[wid][d] : 0;
         rank[r] = before + __popc(peers & lanemask_lt());
         __syncwarp();
@@ -647,6 +650,186 @@ rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **id
     *keys = kin;
     *idx = iin;
     return cuda_check(c, cudaGetLastError(), "radix sort");
+}
+
+// ---------------------------------------------------------------------------
+// small builds: bounding cube, keys, sort and gather of one system of up to
+// kSmallSort stars in one block, the keys in shared memory over the seven passes
+// (one tile, so a pass needs no look-back). The nine launches of the general path
+// are mostly latency: build of 1000 stars 104 -> 58 us, of 4096 117 -> 87; at
+// 8192 one SM's rate is what counts (130 against 124 us). The keys, their order
+// and the cube are the same bits.
+// ---------------------------------------------------------------------------
+constexpr int64_t kSmallSort = 4096;
+constexpr int kSmallThreads = 512, kSmallWarps = kSmallThreads / 32;
+
+struct SmallArgs {
+    int n;
+    const float *x, *y, *z, *mass;
+    double *mbounds;
+    int *mroot;
+    unsigned *zero;   // the words later kernels count in
+    int64_t nzero;
+    uint64_t *key_out;
+    int *perm;
+    float4 *pos;
+    DevState *st;
+};
+
+template <int ITEMS>
+struct SmallSmem {
+    uint64_t key[2][kSmallThreads * ITEMS];
+    unsigned short idx[2][kSmallThreads * ITEMS];
+    unsigned short cnt[kSmallWarps][kSortBins];
+    int lstart[kSortBins];
+    int sw[32];
+    float red[6][kSmallWarps];
+    double bounds[5];
+};
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kSmallThreads) small_sort_k(SmallArgs A) {
+    extern __shared__ __align__(16) char small_smem[];
+    SmallSmem<ITEMS> &S = *reinterpret_cast<SmallSmem<ITEMS> *>(small_smem);
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, n = A.n;
+    for (int64_t i = t; i < A.nzero; i += kSmallThreads) A.zero[i] = 0;
+    // element r of a thread: the warp's consecutive elements in rounds of 32
+    const int base = wid * (32 * ITEMS) + lane;
+    float px[ITEMS], py[ITEMS], pz[ITEMS];
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = base + r * 32;
+        if (i < n) {
+            px[r] = A.x[i];
+            py[r] = A.y[i];
+            pz[r] = A.z[i];
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++)
+        if (base + r * 32 < n) {
+            lo[0] = fminf(lo[0], px[r]); hi[0] = fmaxf(hi[0], px[r]);
+            lo[1] = fminf(lo[1], py[r]); hi[1] = fmaxf(hi[1], py[r]);
+            lo[2] = fminf(lo[2], pz[r]); hi[2] = fmaxf(hi[2], pz[r]);
+        }
+    auto warp_minmax = [&]() {
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            for (int o = 16; o > 0; o >>= 1) {
+                lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+                hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+            }
+    };
+    warp_minmax();
+    if (lane == 0)
+        for (int a = 0; a < 3; a++) {
+            S.red[a][wid] = lo[a];
+            S.red[3 + a][wid] = hi[a];
+        }
+    __syncthreads();
+    if (wid == 0) {
+        for (int a = 0; a < 3; a++) {
+            lo[a] = S.red[a][lane % kSmallWarps];
+            hi[a] = S.red[3 + a][lane % kSmallWarps];
+        }
+        warp_minmax();
+        if (lane == 0) {
+            cube_of(lo, hi, S.bounds);
+            for (int k = 0; k < 5; k++) A.mbounds[k] = A.st->bounds[k] = S.bounds[k];
+            A.mroot[0] = -1;
+        }
+    }
+    __syncthreads();
+    const GridAxis gx = grid_axis(S.bounds[0], S.bounds[4]), gy = grid_axis(S.bounds[1], S.bounds[4]),
+                   gz = grid_axis(S.bounds[2], S.bounds[4]);
+    uint64_t kk[ITEMS];
+    unsigned short ix[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = base + r * 32;
+        kk[r] = i < n ? spread3(grid_coord_fast(px[r], gx)) | (spread3(grid_coord_fast(py[r], gy)) << 1) |
+                            (spread3(grid_coord_fast(pz[r], gz)) << 2)
+                      : 0ull;
+        ix[r] = (unsigned short)i;
+    }
+    for (int p = 0; p < kKeyPasses; p++) {
+        for (int b = lane; b < kSortBins / 2; b += 32) reinterpret_cast<unsigned *>(S.cnt[wid])[b] = 0;
+        if (p > 0) {
+#pragma unroll
+            for (int r = 0; r < ITEMS; r++) {
+                const int i = base + r * 32;
+                if (i < n) {
+                    kk[r] = S.key[p & 1][i];
+                    ix[r] = S.idx[p & 1][i];
+                }
+            }
+        }
+        __syncwarp();
+        unsigned short rank[ITEMS];
+#pragma unroll
+        for (int r = 0; r < ITEMS; r++) {
+            const bool ok = base + r * 32 < n;
+            const int d = ok ? (int)(kk[r] >> (p * kSortBits)) & (kSortBins - 1) : kSortBins;
+            const unsigned peers = match_digit(d, ok);
+            const int before = ok ? S.cnt[wid][d] : 0;
+            rank[r] = (unsigned short)(before + __popc(peers & lanemask_lt()));
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) S.cnt[wid][d] = (unsigned short)(before + __popc(peers));
+            __syncwarp();
+        }
+        __syncthreads();
+        // digits 2t, 2t + 1 (t < 256), two 16-bit counts a word (they stay below 2^16
+        // together): the warps' counts become offsets in the runs; then the runs' starts
+        unsigned tot = 0;
+        if (t < kSortBins / 2) {
+            unsigned v[kSmallWarps];
+#pragma unroll
+            for (int w = 0; w < kSmallWarps; w++) v[w] = reinterpret_cast<unsigned *>(S.cnt[w])[t];
+#pragma unroll
+            for (int w = 0; w < kSmallWarps; w++) {
+                reinterpret_cast<unsigned *>(S.cnt[w])[t] = tot;
+                tot += v[w];
+            }
+        }
+        int total;
+        const int t0 = (int)(tot & 0xffffu), ex = block_exclusive_scan<kSmallThreads>(t0 + (int)(tot >> 16), S.sw, total);
+        if (t < kSortBins / 2) {
+            S.lstart[2 * t] = ex;
+            S.lstart[2 * t + 1] = ex + t0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; r++)
+            if (base + r * 32 < n) {
+                const int d = (int)(kk[r] >> (p * kSortBits)) & (kSortBins - 1);
+                const int slot = S.lstart[d] + S.cnt[wid][d] + rank[r];
+                S.key[(p + 1) & 1][slot] = kk[r];
+                S.idx[(p + 1) & 1][slot] = ix[r];
+            }
+        __syncthreads();
+    }
+    constexpr int last = kKeyPasses & 1;
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+        const int i = r * kSmallThreads + t;
+        if (i < n) {
+            const int j = S.idx[last][i];
+            A.key_out[i] = S.key[last][i];
+            A.perm[i] = j;
+            A.pos[i] = make_float4(A.x[j], A.y[j], A.z[j], A.mass[j]);
+        }
+    }
+}
+
+template <int ITEMS>
+static rv_status small_sort(rv_ctx *c, const SmallArgs &A, cudaStream_t s) {
+    auto kern = small_sort_k<ITEMS>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<ITEMS>));
+    if (e != cudaSuccess) return cuda_check(c, e, "small sort");
+    kern<<<1, kSmallThreads, sizeof(SmallSmem<ITEMS>), s>>>(A);
+    count_launch(c);
+    return cuda_check(c, cudaGetLastError(), "small sort");
 }
 
 // ---------------------------------------------------------------------------
@@ -1151,28 +1334,37 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
         if (r == RV_OK) c->built = true;
         return r;
     }
-    // bounds and keys: blocks per member sized by the largest member
     const int nblk = ceil_div(n, kTopoBlock);
     // cells a tile of the groups pass (few in small builds: more blocks); cleared
     // first: tickets, digit counts, the look-back words of the topology scan and of that pass
     const int tc = n < (1 << 19) ? 64 : 256;
     const int64_t nzero = kLbGroups(c->n_max) + 2 + ceil_div(c->cell_cap, tc);
-    const int bpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, kBoundsChunk), 512 / M + 1));
-    bounds_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, x, y, z, w.bpart, w.barrive, w.mbounds, w.st, w.lb, nzero,
-                                          w.mroot);
-    count_launch(c);
-    // (each block adds its digit counts to the global ones: at least 1024 stars a block)
-    const int kpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, 1024), (int64_t)c->num_sms * 8 / M + 1));
-    // the packed stars live in the group records' space until the gather: the
-    // groups are written after it (32 B per star of room there, 16 needed)
-    float4 *xyzm = reinterpret_cast<float4 *>(w.groups);
-    const int64_t tiles = ceil_div(n, kSortThreads * sort_items(n));
-    keys_k<<<dim3(kpm, M), 256, 0, s>>>(w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm, w.lb + kLbHist,
-                                        reinterpret_cast<uint4 *>(w.words[0]), tiles * kSortBins / 4);
-    count_launch(c);
     uint64_t *skey;
     int *perm;
-    if ((r = radix_sort(c, n, kKeyPasses, &skey, &perm, s, true, true, xyzm, w.pos)) != RV_OK) return r;
+    if (M == 1 && n <= kSmallSort) {
+        skey = w.key_a;
+        perm = w.idx_a;
+        const SmallArgs A{(int)n, x, y, z, m, w.mbounds, w.mroot, w.lb, nzero, skey, perm, w.pos, w.st};
+        static_assert(kSmallSort <= 8 * kSmallThreads, "a thread's share");
+        r = n <= 2 * kSmallThreads ? small_sort<2>(c, A, s) : small_sort<8>(c, A, s);
+        if (r != RV_OK) return r;
+    } else {
+        // bounds and keys: blocks per member sized by the largest member
+        const int bpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, kBoundsChunk), 512 / M + 1));
+        bounds_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, x, y, z, w.bpart, w.barrive, w.mbounds, w.st, w.lb, nzero,
+                                              w.mroot);
+        count_launch(c);
+        // (each block adds its digit counts to the global ones: at least 1024 stars a block)
+        const int kpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, 1024), (int64_t)c->num_sms * 8 / M + 1));
+        // the packed stars live in the group records' space until the gather: the
+        // groups are written after it (32 B per star of room there, 16 needed)
+        float4 *xyzm = reinterpret_cast<float4 *>(w.groups);
+        const int64_t tiles = ceil_div(n, kSortThreads * sort_items(n));
+        keys_k<<<dim3(kpm, M), 256, 0, s>>>(w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm, w.lb + kLbHist,
+                                            reinterpret_cast<uint4 *>(w.words[0]), tiles * kSortBins / 4);
+        count_launch(c);
+        if ((r = radix_sort(c, n, kKeyPasses, &skey, &perm, s, true, true, xyzm, w.pos)) != RV_OK) return r;
+    }
     w.skey = skey;
     w.perm = perm;
     // topology

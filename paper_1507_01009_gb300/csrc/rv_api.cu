@@ -94,16 +94,17 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.pflag = (uint8_t *)take(n);
     t.red = (double *)take(8 * 9 * kRedSlots);
     t.sel_flag = (int *)take(4 * n);
-    t.selhist = (int *)take(4 * (size_t)kMaxMembers * kSelBins);
-    t.selcand = (int *)take(4 * kMaxMembers);
     t.moff = (int64_t *)take(8 * (kMaxMembers + 1));
     t.mbounds = (double *)take(8 * 5 * kMaxMembers);
     t.mroot = (int *)take(4 * kMaxMembers);
     t.bpart = (float *)take(4 * 6 * 2048);
-    t.barrive = (int *)take(4 * kMaxMembers);
     t.xmem = (int *)take(4 * kExtraTotal);
     t.npert = (int *)take(4 * kMaxMembers);
     t.gstack = (int *)take(4 * (size_t)kStackSpillWarps * kStackSpill);
+    // zero when the workspace is set, kept so by what uses them: side by side, one clear
+    t.selhist = (int *)take(4 * (size_t)kMaxMembers * kSelBins);
+    t.selcand = (int *)take(4 * kMaxMembers);
+    t.barrive = (int *)take(4 * kMaxMembers);
     t.st = (DevState *)take(sizeof(DevState));
     if (w) *w = t;
     return off;
@@ -209,10 +210,8 @@ rv_status rv_set_workspace(rv_ctx *c, void *dev, size_t bytes) {
         cudaGraphExecDestroy(c->graph);
         c->graph = nullptr;
     }
-    cudaError_t e = cudaMemset(c->w.st, 0, sizeof(DevState));
-    if (e == cudaSuccess) e = cudaMemset(c->w.barrive, 0, 4 * kMaxMembers);
-    if (e == cudaSuccess) e = cudaMemset(c->w.selhist, 0, 4 * (size_t)kMaxMembers * kSelBins);
-    if (e == cudaSuccess) e = cudaMemset(c->w.selcand, 0, 4 * kMaxMembers);
+    char *clear = reinterpret_cast<char *>(c->w.selhist), *end = reinterpret_cast<char *>(c->w.st + 1);
+    cudaError_t e = cudaMemset(clear, 0, (size_t)(end - clear));
     return cuda_check(c, e, "workspace init");
 }
 

@@ -17,9 +17,11 @@ def rvmod():
     return rv
 
 
-# sort tiles of 1024, 2048 and 4096 change at 2^17 and 2^18 stars; n_leaf 1 gives
+# one block sorts up to 1024 and up to 4096 stars, then tiles of 1024; tiles of
+# 2048 and 4096 from 2^17 and 2^18 stars; n_leaf 1 gives
 # the most cells (many group tiles), n_leaf 64 the fewest
-@pytest.mark.parametrize("n,n_leaf,G", [(2, 1, 1), (1024, 1, 3), (1025, 64, 64), (8191, 1, 1), ((1 << 17) - 1, 24, 64),
+@pytest.mark.parametrize("n,n_leaf,G", [(2, 1, 1), (31, 4, 4), (1023, 1, 3), (1024, 8, 32), (1025, 64, 64), (4095, 2, 7),
+                                        (4096, 1, 1), (4097, 16, 32), (8191, 1, 1), ((1 << 17) - 1, 24, 64),
                                         (1 << 17, 4, 8), ((1 << 18) - 1, 64, 64), ((1 << 18) + 4097, 16, 32),
                                         ((1 << 19) + 1, 24, 64)])
 def test_tree_bits_at_tile_edges(rvmod, n, n_leaf, G):
