@@ -237,7 +237,8 @@ __global__ void __launch_bounds__(256) near_gather_k(SelNear A) {
     });
 }
 
-__global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
+template <int NT>
+__global__ void __launch_bounds__(NT) near_sort_k(SelNear A) {
     extern __shared__ __align__(16) char near_smem[];
     uint64_t *v = reinterpret_cast<uint64_t *>(near_smem);   // [kSelCap]
     __shared__ int h[kSelBins], sw[32], found[2], nacc, nrem;
@@ -248,21 +249,21 @@ __global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
     const int take = (int)min((int64_t)A.k, e - s);
     int rem = take > 0 ? A.ncand[m] : 0, acc = 0;
     __syncthreads();
-    for (int b = t; b < kSelBins; b += 1024) hist[b] = 0;   // ready for the next selection
+    for (int b = t; b < kSelBins; b += NT) hist[b] = 0;   // ready for the next selection
     if (t == 0) {
         A.ncand[m] = 0;
         nacc = 0;
     }
     uint64_t *a = A.cand + s, *o = A.alt + s;
     for (int shift = 53; acc + rem > kSelCap; shift = max(shift - 11, 0)) {
-        for (int b = t; b < kSelBins; b += 1024) h[b] = 0;
+        for (int b = t; b < kSelBins; b += NT) h[b] = 0;
         if (t == 0) nrem = 0;
         __syncthreads();
-        for (int i = t; i < rem; i += 1024) atomicAdd(&h[(int)(a[i] >> shift) & (kSelBins - 1)], 1);
+        for (int i = t; i < rem; i += NT) atomicAdd(&h[(int)(a[i] >> shift) & (kSelBins - 1)], 1);
         __syncthreads();
         int bin, before;
-        find_bin<1024>(h, take - acc, sw, found, bin, before);
-        for (int i = t; i < rem; i += 1024) {
+        find_bin<NT>(h, take - acc, sw, found, bin, before);
+        for (int i = t; i < rem; i += NT) {
             const uint64_t w = a[i];
             const int d = (int)(w >> shift) & (kSelBins - 1);
             if (d < bin) v[atomicAdd(&nacc, 1)] = w;          // among the k nearest: at most take of these
@@ -276,14 +277,16 @@ __global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
         o = q;
         __syncthreads();
     }
-    for (int i = t; i < rem; i += 1024) v[acc + i] = a[i];
+    for (int i = t; i < rem; i += NT) v[acc + i] = a[i];
     int size = 2;
     while (size < acc + rem) size <<= 1;
-    for (int i = acc + rem + t; i < size; i += 1024) v[i] = ~0ull;
-    for (int k = 2; k <= size; k <<= 1)   // bitonic sort
+    for (int i = acc + rem + t; i < size; i += NT) v[i] = ~0ull;
+    __syncthreads();
+    // bitonic sort; pairs up to 32 apart stay within a warp's 64 elements, so only
+    // longer strides, and the step from one back to them, need the block's barrier
+    for (int k = 2; k <= size; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            __syncthreads();
-            for (int q = t; q < size / 2; q += 1024) {
+            for (int q = t; q < size / 2; q += NT) {
                 const int i = 2 * q - (q & (j - 1));   // the pair's lower place
                 const uint64_t lo = v[i], hi = v[i + j];
                 if ((lo > hi) == ((i & k) == 0)) {
@@ -291,10 +294,12 @@ __global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
                     v[i + j] = lo;
                 }
             }
+            if (j > 32 || (j == 1 && k >= 64)) __syncthreads();
+            else __syncwarp();
         }
     __syncthreads();
     const int kk = min(take, A.cap);
-    for (int i = t; i < kk; i += 1024) A.idx[ch * A.cap + i] = (int)(unsigned)v[i];
+    for (int i = t; i < kk; i += NT) A.idx[ch * A.cap + i] = (int)(unsigned)v[i];
     if (t == 0) {
         A.count[ch] = kk;
         if (A.report) A.st->n_pert = kk;
@@ -304,13 +309,17 @@ __global__ void __launch_bounds__(1024) near_sort_k(SelNear A) {
 
 static rv_status select_nearest(rv_ctx *c, const SelNear &A, int members, int64_t largest, cudaStream_t s) {
     const size_t smem = sizeof(uint64_t) * kSelCap;
-    cudaError_t e = cudaFuncSetAttribute(near_sort_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (few candidates: a small block, whose barriers are cheaper)
+    const bool few = std::min(A.k, A.cap) <= 512;
+    cudaError_t e = few ? cudaFuncSetAttribute(near_sort_k<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                        : cudaFuncSetAttribute(near_sort_k<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(c, e, "select nearest");
     // about 1024 stars a block, four blocks an SM over all members
     const int bx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(largest, 1024), (int64_t)c->num_sms * 4 / members + 1));
     near_hist_k<<<dim3(bx, members), 256, 0, s>>>(A);
     near_gather_k<<<dim3(bx, members), 256, 0, s>>>(A);
-    near_sort_k<<<members, 1024, smem, s>>>(A);
+    if (few) near_sort_k<256><<<members, 256, smem, s>>>(A);
+    else near_sort_k<1024><<<members, 1024, smem, s>>>(A);
     c->launches += 3;
     return cuda_check(c, cudaGetLastError(), "select nearest");
 }
@@ -554,11 +563,19 @@ template <int NT>
 __device__ void block_sum4(double v[4], double (*sm)[NT]) {
     for (int a = 0; a < 4; a++) sm[a][threadIdx.x] = v[a];
     __syncthreads();
-    for (int o = NT / 2; o > 0; o >>= 1) {
+    for (int o = NT / 2; o >= 32; o >>= 1) {
         if ((int)threadIdx.x < o)
             for (int a = 0; a < 4; a++) sm[a][threadIdx.x] += sm[a][threadIdx.x + o];
         __syncthreads();
     }
+    if (threadIdx.x < 32) {   // the last five halvings within a warp
+        for (int a = 0; a < 4; a++) {
+            double s = sm[a][threadIdx.x];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (threadIdx.x == 0) sm[a][0] = s;
+        }
+    }
+    __syncthreads();
     for (int a = 0; a < 4; a++) v[a] = sm[a][0];
     __syncthreads();
 }
@@ -719,6 +736,36 @@ __global__ void chain_accel_k(int M, int n_ch, const double *cm, const double *c
     }
 }
 
+// Prediction and pull in one launch, for chains of few members (each block
+// predicts the perturbers for itself; the operations are those of predict_pert_k
+// and pert_on_members_k). A substep of a pair with 256 perturbers is two short
+// kernels otherwise: 12 us a call, 7 in one.
+constexpr int kPredictFused = 8;   // members of a chain up to which predicting again costs less than a launch
+__global__ void __launch_bounds__(256) predict_on_members_k(int n_ch, int cap, const int *idx, const int *npert,
+                                                            const float *x, const float *y, const float *z,
+                                                            const float *vx, const float *vy, const float *vz,
+                                                            const float *m, double dt, const double *cx, double *a_chain,
+                                                            double *pot_chain) {
+    __shared__ double sm[4][256];
+    const int mb = blockIdx.y;
+    const int np = min(npert[mb], cap);
+    const int64_t kk = (int64_t)mb * n_ch + blockIdx.x;
+    const double px = cx[3 * kk], py = cx[3 * kk + 1], pz = cx[3 * kk + 2];
+    double v[4] = {0, 0, 0, 0};
+    for (int p = threadIdx.x; p < np; p += 256) {
+        const int i = idx[(int64_t)mb * cap + p];
+        const double qx = __dadd_rn((double)x[i], __dmul_rn((double)vx[i], dt));
+        const double qy = __dadd_rn((double)y[i], __dmul_rn((double)vy[i], dt));
+        const double qz = __dadd_rn((double)z[i], __dmul_rn((double)vz[i], dt));
+        kep(qx - px, qy - py, qz - pz, (double)m[i], v[0], v[1], v[2], v[3]);
+    }
+    block_sum4<256>(v, sm);
+    if (threadIdx.x == 0) {
+        a_chain[3 * kk] = v[0]; a_chain[3 * kk + 1] = v[1]; a_chain[3 * kk + 2] = v[2];
+        pot_chain[kk] = v[3];
+    }
+}
+
 static const int64_t *system_offsets(const rv_system *sys, int64_t tmp[2]);
 
 // Perturber pull on the chain members at chain positions chain_x (member-major
@@ -728,6 +775,13 @@ rv_status chain_perturber_forces(rv_ctx *c, const rv_system *sys, double dt, con
     Workspace &w = c->w;
     const int M = system_chains(sys);   // the coupling kernels treat each chain as a unit
     const int cap = member_cap(M);
+    if (sys->n_chain <= kPredictFused) {
+        predict_on_members_k<<<dim3(sys->n_chain, M), 256, 0, s>>>(
+            sys->n_chain, cap, w.pert_idx, w.npert, sys->x, sys->y, sys->z, sys->vx, sys->vy, sys->vz, sys->m, dt, chain_x,
+            a_chain, pot_chain ? pot_chain : w.chain_ext_pot);
+        count_launch(c);
+        return cuda_check(c, cudaGetLastError(), "chain perturber forces");
+    }
     predict_pert_k<<<dim3(ceil_div(cap, 128), M), 128, 0, s>>>(cap, w.pert_idx, w.npert, sys->x, sys->y, sys->z,
                                                                sys->vx, sys->vy, sys->vz, sys->m, dt, w.pert_m,
                                                                w.pert_x);
@@ -899,6 +953,22 @@ constexpr int kRedQ = 9;  // ekin, epot, P(3), L(3), mass
 
 static int energy_bpm(int M) { return std::max(1, std::min(256, kRedSlots / M)); }
 
+// Tree sums of kRedQ rows of 256 (o = 128 .. 1, element t + o onto t) into column
+// 0: the strides below a warp by shuffles, one row a warp, the same pairs.
+__device__ __forceinline__ void red_tree(double (*sm)[256]) {
+    for (int o = 128; o >= 32; o >>= 1) {
+        if ((int)threadIdx.x < o)
+            for (int a = 0; a < kRedQ; a++) sm[a][threadIdx.x] += sm[a][threadIdx.x + o];
+        __syncthreads();
+    }
+    for (int a = threadIdx.x >> 5; a < kRedQ; a += 8) {
+        double s = sm[a][threadIdx.x & 31];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) sm[a][0] = s;
+    }
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(256) energy_partial_k(const int64_t *moff, int bpm, const float *x, const float *y,
                                                         const float *z, const float *vx, const float *vy,
                                                         const float *vz, const float *m, const float *pot,
@@ -916,11 +986,7 @@ __global__ void __launch_bounds__(256) energy_partial_k(const int64_t *moff, int
     }
     for (int a = 0; a < kRedQ; a++) sm[a][threadIdx.x] = q[a];
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            for (int a = 0; a < kRedQ; a++) sm[a][threadIdx.x] += sm[a][threadIdx.x + o];
-        __syncthreads();
-    }
+    red_tree(sm);
     if (threadIdx.x < kRedQ) part[kRedQ * ((int64_t)mb * bpm + blockIdx.x) + threadIdx.x] = sm[threadIdx.x][0];
 }
 
@@ -932,11 +998,7 @@ __global__ void __launch_bounds__(256) energy_final_k(const double *part, int bp
     for (int a = 0; a < kRedQ; a++)
         sm[a][threadIdx.x] = ((int)threadIdx.x < bpm) ? part[kRedQ * ((int64_t)mb * bpm + threadIdx.x) + a] : 0.0;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            for (int a = 0; a < kRedQ; a++) sm[a][threadIdx.x] += sm[a][threadIdx.x + o];
-        __syncthreads();
-    }
+    red_tree(sm);
     if (threadIdx.x == 0) {
         double q[kRedQ];
         for (int a = 0; a < kRedQ; a++) q[a] = sm[a][0];
