@@ -50,16 +50,21 @@ constexpr int kMaxPert = 5000;
 // of 4096, 8192, 16384, 32768: 719, 614, 562, 643 / 1832, 1703, 1660, 1676;
 // unsplit 1286 / 1801.
 constexpr int kMaxParts = 16;
-constexpr int kPartItems = 16384;
+// A single system of 2^17 to 2^19 stars takes twice as many: its full walks change
+// by -2 to +1 % (131072 stars 1105 -> 1086 us, 200001 1647 -> 1665), and the walks of
+// block time steps, in which few groups are active, by a quarter (sixteen
+// substeps of 200001 stars 12.4 -> 10.4 ms); an ensemble of that size loses 3 %.
+constexpr int kPartItems = 16384, kPartItemsMid = 2 * kPartItems;
 // Cells of more than 1 / kPartGrain of their member's stars are traversed by
 // every part (Part in walk.cu). Smaller subtrees balance better, larger ones
 // repeat less: 16000 / 65536 / 200001 stars took 169 / 593 / 1698 us at 32,
 // 150 / 562 / 1660 at 64, 158 / 581 / 1672 at 128, 172 / 589 / 1664 at 256.
 constexpr int kPartGrain = 64;
-__host__ __device__ __forceinline__ int parts_of(int64_t n, int group) {
+inline int parts_of(int64_t n, int members, int group) {
     const int64_t g = n / group + 1;
+    const int64_t items = members == 1 && n >= (1 << 17) && n < (1 << 19) ? kPartItemsMid : kPartItems;
     int P = 1;
-    while (P < kMaxParts && 2 * P * g <= kPartItems) P <<= 1;
+    while (P < kMaxParts && 2 * P * g <= items) P <<= 1;
     return P;
 }
 // of a group with `count` stars: at most one part a star, so that the items are at most n

@@ -46,8 +46,9 @@
 // warp per block; 112 registers a thread (the running sums and what a work item
 // needs at its end live in shared memory) give 16 warps per SM, as 104 and 128
 // do, and nothing spills. Walk of 2^20 stars at theta 0.5 / 2^22 at 0.8, tile 96:
-// 8.50 / 18.3 ms at 112, 8.69 / 18.8 at 104, 9.07 / 19.7 at 120, 9.2 / 19.9 at
-// 128; cell pairs 2, 3, 4 at 112: 8.86, 8.52, 8.50 ms.
+// 8.44 / 18.2 ms at 112, 8.60 / 18.7 at 104, 9.07 / 19.7 at 120, 9.2 / 19.9 at
+// 128; cell pairs 2, 3, 4, 6, 8 at 112: 8.86, 8.52, 8.44, 8.36, 8.36 ms, but 65536
+// stars (short tiles, two copies of the loop in use) 541 us at 4, 570 at 6, 619 at 8.
 #ifndef RV_P2P_UNROLL
 #define RV_P2P_UNROLL 1
 #endif
@@ -211,24 +212,22 @@ struct Tgt {
     int j0, k;
 };
 
-// A lane's running sums for its two targets, kept in the warp's shared
-// memory (not registers, which the evaluation loops need): for target q,
-// field k = ax, ay, az, ph, then their Neumaier compensations (k + 4), at
-// word (q * 8 + k) * 32 + lane, so the 32 lanes touch 32 consecutive words.
+// A lane's running sums for its two targets, kept in the warp's shared memory
+// (not registers, which the evaluation loops need): for target q the sums (ax,
+// ay, az, ph) at float4 2 q * 32 + lane, their Neumaier compensations at (2 q +
+// 1) * 32 + lane, so a tile's sums take eight 16-byte accesses of consecutive lanes.
 struct AccSm {
-    float *p;   // the warp's region + lane
-    __device__ __forceinline__ float &f(int q, int k) const { return p[(q * 8 + k) * 32]; }
+    float4 *p;   // the warp's region + lane
 };
 
 __device__ __forceinline__ void add_tile(const AccSm &A, int q, f2 tx, f2 ty, f2 tz, f2 tp) {
-    const float v[4] = {f2_sum(tx), f2_sum(ty), f2_sum(tz), -f2_sum(tp)};
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        float sum = A.f(q, k), comp = A.f(q, k + 4);
-        nadd(sum, comp, v[k]);
-        A.f(q, k) = sum;
-        A.f(q, k + 4) = comp;
-    }
+    float4 s = A.p[2 * q * 32], c = A.p[(2 * q + 1) * 32];
+    nadd(s.x, c.x, f2_sum(tx));
+    nadd(s.y, c.y, f2_sum(ty));
+    nadd(s.z, c.z, f2_sum(tz));
+    nadd(s.w, c.w, -f2_sum(tp));
+    A.p[2 * q * 32] = s;
+    A.p[(2 * q + 1) * 32] = c;
 }
 
 // Spline softening (the "spline" option of Sect. 2): the point mass smoothed
@@ -459,13 +458,19 @@ __device__ __forceinline__ void move_front(float4 *list, int from, int mv) {
     const int lane = threadIdx.x & 31;
     const float4 *src = list + F4 * (from + lane);
     float4 *dst = list + F4 * lane;
+    if (from >= 32) {
+        if (lane < mv) {
 #pragma unroll
-    for (int f = 0; f < F4; f++) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (lane < mv) v = src[f];
-        if (from < 32) __syncwarp();
-        if (lane < mv) dst[f] = v;
-        if (from < 32) __syncwarp();
+            for (int f = 0; f < F4; f++) dst[f] = src[f];
+        }
+    } else {
+        for (int f = 0; f < F4; f++) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane < mv) v = src[f];
+            __syncwarp();
+            if (lane < mv) dst[f] = v;
+            __syncwarp();
+        }
     }
     __syncwarp();
 }
@@ -777,9 +782,9 @@ __device__ __forceinline__ bool walk_group(const WalkArgs &A, const TreeGeo &G, 
 }
 
 // Zeroes the warp's running sums.
-__device__ __forceinline__ void clear_acc(float *accw) {
+__device__ __forceinline__ void clear_acc(float4 *accw) {
 #pragma unroll
-    for (int k = 0; k < 16; k++) accw[32 * k + (threadIdx.x & 31)] = 0.f;
+    for (int k = 0; k < 4; k++) accw[32 * k + (threadIdx.x & 31)] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();
 }
 
@@ -787,7 +792,7 @@ __device__ __forceinline__ void clear_acc(float *accw) {
 // l / p; the k lanes t, t + p, ..., t + (k - 1) p of a pair add their partial
 // totals in that order, read from the warp's running sums (AccSm). Returns the
 // totals of stars `lane` and `lane + 32`.
-__device__ __forceinline__ void combine_shares(const float *accw, int s, int p, int k, Acc out[2]) {
+__device__ __forceinline__ void combine_shares(const float4 *accw, int s, int p, int k, Acc out[2]) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
 #pragma unroll
@@ -796,10 +801,11 @@ __device__ __forceinline__ void combine_shares(const float *accw, int s, int p, 
         Acc o = {};
         if (i < s)
             for (int m = 0; m < k; m++) {
-                const float *e = accw + (i & 1) * 8 * 32 + (i >> 1) + m * p;
-                nadd(o.ax, o.cx, e[0]); nadd(o.ay, o.cy, e[32]);
-                nadd(o.az, o.cz, e[64]); nadd(o.ph, o.cp, e[96]);
-                o.cx += e[128]; o.cy += e[160]; o.cz += e[192]; o.cp += e[224];
+                const float4 *e = accw + (i & 1) * 64 + (i >> 1) + m * p;
+                const float4 v = e[0], w = e[32];
+                nadd(o.ax, o.cx, v.x); nadd(o.ay, o.cy, v.y);
+                nadd(o.az, o.cz, v.z); nadd(o.ph, o.cp, v.w);
+                o.cx += w.x; o.cy += w.y; o.cz += w.z; o.cp += w.w;
             }
         out[h] = o;
     }
@@ -910,7 +916,7 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
         if (lane == 0) gi = atomicAdd(&A.st->walk.next_item, 1);
         gi = __shfl_sync(0xffffffffu, gi, 0);
         if (gi >= nitem) break;
-        float *accw = reinterpret_cast<float *>(wsm + warp_staging_bytes(A.tile));
+        float4 *accw = reinterpret_cast<float4 *>(wsm + warp_staging_bytes(A.tile));
         const AccSm acc{accw + lane};
         unsigned a2 = 0, a3 = 0;   // list entries of the group: stars, cells
         if (gi < A.n_extra) {
@@ -1247,7 +1253,7 @@ rv_status tree_walk(rv_ctx *c, float theta, float eps_star, int n_extra, const f
     A.opart = w.gopart;
     A.scost = w.scost;
     A.n_leaf = c->cfg.n_leaf;
-    A.parts = parts_of(c->n, c->cfg.group);
+    A.parts = parts_of(c->n, c->n_members, c->cfg.group);
     A.partial = w.gpartial;
     A.garrive = w.garrive;
     const bool spline = c->cfg.softening == 1 && eps_star > 0.f;

@@ -20,9 +20,10 @@ def rvmod():
     return rv
 
 
-def last_n(P, group):
-    """The largest build walked in P parts: P (n / group + 1) <= 16384 (integer division)."""
-    return (16384 // P) * group - 1
+def last_n(P, group, items=16384):
+    """The largest build walked in P parts: P (n / group + 1) <= items (integer division); items doubles for a
+    single system of 2^17 to 2^19 stars."""
+    return (items // P) * group - 1
 
 
 # one star, groups smaller than the parts, both sides of 16 / 8 parts (groups of 1, 7, 32 and 64 stars), a ragged middle
@@ -46,7 +47,7 @@ def test_split_walk_vs_oracle(rvmod, n, group, n_leaf, quad):
         assert med <= MED_TOL and mx <= MAX_TOL, (med, mx)
 
 
-@pytest.mark.parametrize("n", [last_n(8, 64), last_n(4, 64) + 1])
+@pytest.mark.parametrize("n", [last_n(8, 64), last_n(8, 64) + 1, last_n(8, 64, 32768) + 1])
 def test_split_walk_repeats_and_masks(rvmod, n):
     """Cost-ordered, volume-ordered and masked walks of a split build give the same bits."""
     import torch
