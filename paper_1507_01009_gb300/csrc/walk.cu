@@ -49,11 +49,20 @@
 // 8.44 / 18.2 ms at 112, 8.60 / 18.7 at 104, 9.07 / 19.7 at 120, 9.2 / 19.9 at
 // 128; cell pairs 2, 3, 4, 6, 8 at 112: 8.86, 8.52, 8.44, 8.36, 8.36 ms, but 65536
 // stars (short tiles, two copies of the loop in use) 541 us at 4, 570 at 6, 619 at 8.
+// Under spline softening the loops carry a branch per pair and the code of an
+// unrolled cell loop no longer stays in the instruction cache beside the star loop:
+// cell pairs 1, 2, 3, 4 there take 11.01, 10.82, 10.99, 11.77 ms on 2^20 stars
+// (theta 0.5, groups of 64), 11.63, 11.52, 12.30, 13.81 in groups of 32, 7.15, 7.86,
+// 9.09, 10.01 under the relative criterion in groups of 32, and 1.14, 1.31, 1.54,
+// 1.68 on 100003 stars; one it is.
 #ifndef RV_P2P_UNROLL
 #define RV_P2P_UNROLL 1
 #endif
 #ifndef RV_M2P_UNROLL
 #define RV_M2P_UNROLL 4
+#endif
+#ifndef RV_M2P_UNROLL_SPLINE
+#define RV_M2P_UNROLL_SPLINE 1
 #endif
 #ifndef RV_WALK_MAXNREG
 #define RV_WALK_MAXNREG 112
@@ -132,7 +141,7 @@ struct WalkArgs {
 // pair: (x, y), (z, m). Running sums: 16 floats per lane (AccSm).
 constexpr int kCellPairF4 = 5, kStarPairF4 = 2;
 constexpr int kAccWords = 16 * 32;
-constexpr int kP2PUnroll = RV_P2P_UNROLL, kM2PUnroll = RV_M2P_UNROLL;
+constexpr int kP2PUnroll = RV_P2P_UNROLL, kM2PUnroll = RV_M2P_UNROLL, kM2PUnrollSpline = RV_M2P_UNROLL_SPLINE;
 __host__ __device__ inline size_t warp_staging_bytes(int tile) {
     return (size_t)kStackSm * 4 + 64 * 4 + (size_t)(tile + 64) / 2 * 16 * kCellPairF4 +
            (size_t)(tile + 64) / 2 * 16 * kStarPairF4;
@@ -326,7 +335,7 @@ __device__ __forceinline__ void eval_m2p(const float4 *src, int npair, const Tgt
                                          const AccSm &A) {
     f2 tx[2] = {0, 0}, ty[2] = {0, 0}, tz[2] = {0, 0}, tp[2] = {0, 0};   // tp sums +(M - s/2)/rho
     if (SPL) eps2 = 0;
-#pragma unroll kM2PUnroll
+#pragma unroll(SPL ? kM2PUnrollSpline : kM2PUnroll)
     for (int j = t.j0; j < npair; j += t.k) {
         const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(src) + kCellPairF4 * j;
         const ulonglong2 a = p[0];   // M, cx
