@@ -687,9 +687,9 @@ def build_roofline(ctx, d, S, stream, flush, reps, ms_per_step):
     Algorithmic bytes per build: per star the cube's 12 B read; keys 16 B read
     and 8 B (key) + 16 B (the packed star) written; each of the sort's passes
     (7 of 9 bits for 63-bit keys, one more on the member when there are
-    several) 12 B read + 8 B (the up-sweep's key) + 12 B written; the
-    permutation 4 B + 16 B read and 16 B written; the topology 8 B read; the
-    moments 16 B read; per cell 42 B written by the topology and 48 B read +
+    several) 12 B read + 12 B written; the gather into key order (in the last
+    pass) 16 B read and 16 B written; the topology 8 B read; the moments 16 B
+    read; per cell 42 B written by the topology and 48 B read +
     48 B written by the moments."""
     import torch
     off = d["offsets"] if d["offsets"] is not None else [0, S.n]
@@ -707,12 +707,12 @@ def build_roofline(ctx, d, S, stream, flush, reps, ms_per_step):
     ms = float(np.median([a.elapsed_time(b) for a, b in ev[1:]]))
     n, ncell, _ = ctx.tree_sizes()
     passes = 7 + (1 if len(off) > 2 else 0)
-    per_star = 12 + 40 + passes * 32 + 36 + 8 + 16
+    per_star = 12 + 40 + passes * 24 + 32 + 8 + 16
     nbytes = n * per_star + ncell * (42 + 96)
     gbs = nbytes / (ms / 1e3) / 1e9
     hbm = _measured_peaks().get("hbm_gbs")
     peak = hbm or 6800.0
-    return {"bound": "hbm", "kernels": f"bounds, keys, sort ({passes} passes), gather, topology, groups, moments",
+    return {"bound": "hbm", "kernels": f"bounds, keys (digit counts), sort ({passes} passes, the last gathers), topology, groups and moments",
             "ms": ms, "bytes": float(nbytes), "bytes_per_star": nbytes / max(n, 1), "cells": ncell,
             "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": None,
             "share_of_step": ms / ms_per_step,

@@ -60,7 +60,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *smem_warp, int &
 // below (counts stay under 2^30), so that one store publishes both.
 // ---------------------------------------------------------------------------
 constexpr unsigned kLbSum = 1u << 30, kLbPrefix = 2u << 30, kLbCount = (1u << 30) - 1;
-constexpr int kLbSpins = 1 << 22;   // polls before a wait gives up (seconds)
+constexpr int kLbSpins = 1 << 20;   // polls before a wait gives up (about half a second)
 
 __device__ __forceinline__ unsigned lb_load(const unsigned *p) {
     unsigned v;

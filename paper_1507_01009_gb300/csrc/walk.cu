@@ -45,7 +45,7 @@
 // every tile) and the register budget of the walk kernel. The kernel runs one
 // warp per block; 112 registers a thread (the running sums and what a work item
 // needs at its end live in shared memory) give 16 warps per SM, as 104 and 128
-// do, and nothing spills. Walk of 2^20 stars at theta 0.5 / 2^22 at 0.8, tile 96:
+// do, and 4 bytes spill. Walk of 2^20 stars at theta 0.5 / 2^22 at 0.8, tile 96:
 // 8.44 / 18.2 ms at 112, 8.60 / 18.7 at 104, 9.07 / 19.7 at 120, 9.2 / 19.9 at
 // 128; cell pairs 2, 3, 4, 6, 8 at 112: 8.86, 8.52, 8.44, 8.36, 8.36 ms, but 65536
 // stars (short tiles, two copies of the loop in use) 541 us at 4, 570 at 6, 619 at 8.
