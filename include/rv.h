@@ -446,6 +446,16 @@ rv_status rv_direct_fp64(int64_t n, const double *x, const double *y, const doub
  * gave_up[0] (device int32) = 1 if the wait ran out, else 0. Asynchronous on
  * `stream`; RV_E_INVAL on bad arguments. */
 rv_status rv_wait_selftest(int64_t limit_cycles, int32_t arrive, int32_t *gave_up, void *stream);
+/* Self-test of the bounded look-back waits of the tree build and the searches
+ * (the paper has no counterpart; no GPU fault): arms the context so that the
+ * next launch of `stage` withholds its first tile's sum and every wait in it
+ * gives up after `polls` polls (0 .. 2^20). Stages: 1 .. 8 the passes of a sort
+ * (8: a build's pass over the members), 9 a scan (of a build's cells, or of a
+ * radius, tidal or absorption search), 10 a build's walk groups; 0 disarms. A launch of a single tile
+ * has nothing to wait for. After a wait gave up, rv_sync_status reports
+ * RV_E_TIMEOUT; the tree has no cells or no groups, forces on the stars are not
+ * written, a search selects nothing; the next build or search is whole again. */
+rv_status rv_lookback_selftest(rv_ctx *ctx, int32_t stage, int32_t polls);
 /* Mean squared error of network(x) against t[n][3] and its gradient with
  * respect to the FP32 parameter vector (grad: device FP32 [5768], ordered W1
  * 16x64, b1, W2 64x64, b2, W3 64x8, b3, row-major; loss: device FP32 [1] or

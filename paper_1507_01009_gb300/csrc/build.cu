@@ -55,7 +55,9 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *smem_warp, int &
 // adds up its predecessors' published words back to the nearest full prefix,
 // and publishes its own prefix. A tile's predecessors have always started (the
 // tickets are handed out in order), so every wait ends; waits are bounded all
-// the same, and a block that gives up latches RV_E_TIMEOUT and writes nothing.
+// the same, and a block that gives up latches RV_E_TIMEOUT and writes nothing;
+// what it leaves unwritten is not used: a sort sets the kLbGaveUp word, which the
+// kernels after it read, a scan or the group pass leaves a total of -1.
 // A word holds its state in the top two bits (0: not there yet) and the count
 // below (counts stay under 2^30), so that one store publishes both.
 // ---------------------------------------------------------------------------
@@ -73,14 +75,14 @@ __device__ __forceinline__ void lb_store(unsigned *p, unsigned v) {
 
 // The sum of the tiles before `tile` (one word a tile), by one whole warp: 32
 // predecessors a step. Returns false if a wait gave up.
-__device__ __forceinline__ bool lb_sum_before(const unsigned *words, int tile, unsigned &sum) {
+__device__ __forceinline__ bool lb_sum_before(const unsigned *words, int tile, int polls, unsigned &sum) {
     const int lane = threadIdx.x & 31;
     sum = 0;
     for (int hi = tile - 1; hi >= 0; hi -= 32) {
         const int t = hi - lane;
         unsigned w = t >= 0 ? lb_load(words + t) : kLbPrefix;   // before the first tile: a prefix of 0
         for (int spin = 0; __any_sync(0xffffffffu, (w >> 30) == 0); spin++) {
-            if (spin > kLbSpins) return false;
+            if (spin > polls) return false;
             if ((w >> 30) == 0) w = lb_load(words + t);
         }
         const unsigned pm = __ballot_sync(0xffffffffu, w & kLbPrefix);
@@ -91,16 +93,28 @@ __device__ __forceinline__ bool lb_sum_before(const unsigned *words, int tile, u
     return true;
 }
 
+// The total of a pass by look-back, 0 before the launch: the last tile's sum, or
+// -1 once any tile gave up, in whichever order they end.
+__device__ __forceinline__ void lb_total(int *d_total, bool ok, bool last, int total) {
+    if (!ok) atomicExch(d_total, -1);
+    else if (last) atomicCAS(d_total, 0, total);
+}
+
 // Exclusive scan of int32 (in place), length *d_len (<= nmax) or nmax; the
-// total to *d_total if given. words, ticket: zero before the launch.
+// total to *d_total (lb_total). words, ticket: zero before the launch. gave_up
+// (optional): set if the data is not there, and then nothing is done.
 __global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int *d_len, unsigned *words, int *ticket,
-                                              int *d_total, DevState *st) {
+                                              const unsigned *gave_up, LbWait wait, int *d_total, DevState *st) {
     __shared__ int sw[8], stile;
     __shared__ unsigned sbefore;
     __shared__ bool sok;
-    if (threadIdx.x == 0) stile = atomicAdd(ticket, 1);
+    if (threadIdx.x == 0) {
+        const int t = atomicAdd(ticket, 1);
+        stile = gave_up && lb_load(gave_up) ? -1 : t;
+    }
     __syncthreads();
     const int tile = stile;
+    if (tile < 0) return;
     const int64_t len = d_len ? min((int64_t)*d_len, nmax) : nmax;
     const int64_t base = (int64_t)tile * kScanChunk + threadIdx.x * 8;
     int v[8], s = 0;
@@ -116,15 +130,16 @@ __global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int
     int total;
     const int ex0 = block_exclusive_scan<256>(s, sw, total);
     if (threadIdx.x < 32) {
-        if (threadIdx.x == 0) lb_store(words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
+        if (threadIdx.x == 0 && tile != wait.hold)
+            lb_store(words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
         unsigned before = 0;
-        const bool ok = lb_sum_before(words, tile, before);
+        const bool ok = lb_sum_before(words, tile, wait.polls, before);
         if (threadIdx.x == 0) {
             if (ok && tile) lb_store(words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
             if (!ok) latch_err(st, kErrTimeout);
             sbefore = before;
             sok = ok;
-            if (ok && d_total && tile == (int)gridDim.x - 1) *d_total = (int)before + total;
+            lb_total(d_total, ok, tile == (int)gridDim.x - 1, (int)before + total);
         }
     }
     __syncthreads();
@@ -146,24 +161,30 @@ __global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int
     }
 }
 
+// The wait of a stage's next launch (the self-test's, once, if it named this stage).
+static LbWait lb_wait(rv_ctx *c, int stage) {
+    if (c->lb_test_stage != stage) return LbWait{kLbSpins, -1};
+    c->lb_test_stage = 0;
+    return LbWait{c->lb_test_polls, 0};
+}
+
 static rv_status scan_launch(rv_ctx *c, int *data, int64_t nmax, int *d_total, unsigned *words, int *ticket,
-                             cudaStream_t s) {
-    scan_k<<<ceil_div(nmax, kScanChunk), 256, 0, s>>>(data, nmax, nullptr, words, ticket, d_total, c->w.st);
+                             const unsigned *gave_up, cudaStream_t s) {
+    scan_k<<<ceil_div(nmax, kScanChunk), 256, 0, s>>>(data, nmax, nullptr, words, ticket, gave_up,
+                                                      lb_wait(c, kLbStageScan), d_total, c->w.st);
     count_launch(c);
     return cuda_check(c, cudaGetLastError(), "scan");
 }
 
+// *d_total is 0 before; -1 after it means that a wait gave up.
 rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s) {
-    if (nmax <= 0) {
-        if (d_total) return cuda_check(c, cudaMemsetAsync(d_total, 0, sizeof(int), s), "scan memset");
-        return RV_OK;
-    }
+    if (nmax <= 0) return RV_OK;
     // ticket and words side by side: one clear
     unsigned *z = c->w.lb + kLbScan;
     rv_status r = cuda_check(c, cudaMemsetAsync(z, 0, sizeof(unsigned) * (1 + (size_t)ceil_div(nmax, kScanChunk)), s),
                              "scan");
     if (r != RV_OK) return r;
-    return scan_launch(c, data, nmax, d_total, z + 1, reinterpret_cast<int *>(z), s);
+    return scan_launch(c, data, nmax, d_total, z + 1, reinterpret_cast<int *>(z), nullptr, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -186,7 +207,7 @@ __device__ __forceinline__ void cube_of(const float lo[3], const float hi[3], do
 // Blocks (bx, m): member m's stars, strided by bpm blocks; the last block of a
 // member to finish reduces the blocks' partials (min and max are exact, so the
 // order is free). The first kernel of a build, it also clears the words the
-// later ones count in (zero[nzero]) and the member roots.
+// later ones count in (zero[nzero]), the member roots and the last build's sizes.
 __global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, const float *x, const float *y,
                                                 const float *z, float *part, int *arrive, double *mbounds,
                                                 DevState *st, unsigned *zero, int64_t nzero, int *mroot) {
@@ -194,7 +215,10 @@ __global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, co
     const int64_t nthr = (int64_t)gridDim.x * gridDim.y * 256;
     const int64_t tid = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.x;
     for (int64_t i = tid; i < nzero; i += nthr) zero[i] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) mroot[m] = -1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        mroot[m] = -1;
+        if (m == 0) st->ncell = st->ngroup = 0;
+    }
     const int64_t s = moff[m], e = moff[m + 1];
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int64_t i = s + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (int64_t)bpm * blockDim.x) {
@@ -443,18 +467,23 @@ struct SortSmem {
 template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uint64_t *key_in, const int *idx_in,
                                                             int shift, const int64_t *moff, int M,
-                                                            const unsigned *ghist, int *ticket, unsigned *words,
-                                                            unsigned *words_next, uint64_t *key_out, int *idx_out,
-                                                            const float4 *xyzm, float4 *pos, DevState *st) {
+                                                            const unsigned *ghist, int *ticket, unsigned *gave_up,
+                                                            LbWait wait, unsigned *words, unsigned *words_next,
+                                                            uint64_t *key_out, int *idx_out, const float4 *xyzm,
+                                                            float4 *pos, DevState *st) {
     constexpr int NW = kSortThreads / 32, TILE = kSortThreads * ITEMS;
     static_assert(kSortBins == 2 * kSortThreads, "a thread owns two digits");
     extern __shared__ __align__(16) char sort_smem[];
     SortSmem<ITEMS> &S = *reinterpret_cast<SortSmem<ITEMS> *>(sort_smem);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1);
+    if (threadIdx.x == 0) {
+        const int t = atomicAdd(ticket, 1);
+        S.tile = lb_load(gave_up) ? -1 : t;
+    }
     for (int b = lane; b < kSortBins / 2; b += 32) reinterpret_cast<unsigned *>(S.cnt[wid])[b] = 0;
     __syncthreads();
     const int tile = S.tile;
+    if (tile < 0) return;   // a pass before left slots unwritten: its indices must not be used
     const int64_t tile0 = (int64_t)tile * TILE;
     const int64_t base = tile0 + wid * (32 * ITEMS);
     const int d0 = 2 * threadIdx.x;   // this thread's digits
@@ -502,8 +531,10 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uin
     }
     unsigned *mine = words + (int64_t)tile * kSortBins + d0;
     const unsigned state = tile ? kLbSum : kLbPrefix;
-    lb_store(mine, state | (unsigned)tot0);
-    lb_store(mine + 1, state | (unsigned)tot1);
+    if (tile != wait.hold) {
+        lb_store(mine, state | (unsigned)tot0);
+        lb_store(mine + 1, state | (unsigned)tot1);
+    }
     // digit runs in digit order: exclusive scans of the tile's totals and of the whole input's
     int total;
     const int ex = block_exclusive_scan<kSortThreads>(tot0 + tot1, S.sw, total);
@@ -547,7 +578,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uin
             }
         }
         t -= used;
-        if (used == 0 && ++spin > kLbSpins) {
+        if (used == 0 && ++spin > wait.polls) {
             fail = true;
             break;
         }
@@ -559,7 +590,10 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uin
     S.gbase[d0] = first0 + (int)b0 - ex;
     S.gbase[d0 + 1] = first1 + (int)b1 - (ex + tot0);
     if (__syncthreads_or(fail)) {   // a wait gave up: nothing is written
-        if (threadIdx.x == 0) latch_err(st, kErrTimeout);
+        if (threadIdx.x == 0) {
+            latch_err(st, kErrTimeout);
+            lb_store(gave_up, 1u);
+        }
         return;
     }
 #pragma unroll
@@ -603,13 +637,14 @@ int64_t sort_words(int64_t n_max) {
 
 template <int ITEMS>
 static void sort_pass(rv_ctx *c, int64_t n, const uint64_t *ki, const int *ii, int shift, const int64_t *moff,
-                      const unsigned *ghist, int *ticket, unsigned *words, unsigned *next, uint64_t *ko, int *io,
-                      const float4 *xyzm, float4 *pos, cudaStream_t s) {
+                      const unsigned *ghist, int *ticket, LbWait wait, unsigned *words, unsigned *next, uint64_t *ko,
+                      int *io, const float4 *xyzm, float4 *pos, cudaStream_t s) {
     auto kern = sort_pass_k<ITEMS>;
     if (sizeof(SortSmem<ITEMS>) > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem<ITEMS>));
     kern<<<ceil_div(n, kSortThreads * ITEMS), kSortThreads, sizeof(SortSmem<ITEMS>), s>>>(
-        n, ki, ii, shift, moff, c->n_members, ghist, ticket, words, next, ko, io, xyzm, pos, c->w.st);
+        n, ki, ii, shift, moff, c->n_members, ghist, ticket, c->w.lb + kLbGaveUp, wait, words, next, ko, io, xyzm, pos,
+        c->w.st);
     count_launch(c);
 }
 
@@ -640,7 +675,7 @@ rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **id
         const bool mem = p == passes, lastp = p + 1 == total;
         auto run = items == 4 ? sort_pass<4> : items == 8 ? sort_pass<8> : sort_pass<16>;
         run(c, n, kin, iin, p * kSortBits, mem ? w.moff : nullptr, mem ? nullptr : ghist + p * kSortBins, tickets + p,
-            w.words[p & 1], lastp ? nullptr : w.words[(p + 1) & 1], kout, iout, lastp ? xyzm : nullptr,
+            lb_wait(c, kLbStageSort + p), w.words[p & 1], lastp ? nullptr : w.words[(p + 1) & 1], kout, iout, lastp ? xyzm : nullptr,
             lastp ? pos : nullptr, s);
         // next pass reads what this one wrote
         uint64_t *tk = kin; kin = kout; kout = tk;
@@ -738,6 +773,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_k(SmallArgs A) {
             cube_of(lo, hi, S.bounds);
             for (int k = 0; k < 5; k++) A.mbounds[k] = A.st->bounds[k] = S.bounds[k];
             A.mroot[0] = -1;
+            A.st->ncell = A.st->ngroup = 0;
         }
     }
     __syncthreads();
@@ -930,6 +966,7 @@ __global__ void __launch_bounds__(kTopoBlock) topo_write_k(int64_t n, const uint
     __shared__ int wp[kLevels][kTopoBlock / 32];
     __shared__ int lvoff[kLevels + 1];
     __shared__ int bbase[kLevels + 1];
+    if (st->ncell <= 0) return;   // the sort or the scan gave up: no counts to place cells by
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int64_t i = (int64_t)blockIdx.x * kTopoBlock + threadIdx.x;
     bool valid = i < n;
@@ -958,12 +995,13 @@ __global__ void __launch_bounds__(kTopoBlock) topo_write_k(int64_t n, const uint
     if (blockIdx.x == 0 && threadIdx.x <= kLevels) st->lvoff[threadIdx.x] = lvoff[threadIdx.x];
     if (!valid) return;
     const unsigned lt = lanemask_lt();
+    auto outside = [&](int c) -> bool { return c < 0 || c >= cap; };
     // exclusive global rank of star i among cells of level l
     auto rank = [&](int l) -> int { return bbase[l] + wp[l][wid] + __popc(b.mask[l] & lt); };
     uint64_t k = key[i];
     for (int l = Di; l <= lam; l++) {
         int c = rank(l);
-        if (c >= cap) { latch_err(st, kErrCells); return; }
+        if (outside(c)) { latch_err(st, kErrCells); return; }
         cbox[c] = cell_box(k, l);
         clink[4 * c + 0] = (l < lam) ? rank(l + 1) : 0;  // first child: cell (l + 1, i)
         if (l == lam) clink[4 * c + 1] = 0;
@@ -977,7 +1015,7 @@ __global__ void __launch_bounds__(kTopoBlock) topo_write_k(int64_t n, const uint
         int lp = lamv[i - 1];
         for (int l = Di; l <= lp; l++) {
             int c = rank(l) - 1;
-            if (c >= cap) { latch_err(st, kErrCells); return; }
+            if (outside(c)) { latch_err(st, kErrCells); return; }
             clink[4 * c + 3] = (int)i;
             if (l < lp) clink[4 * c + 1] = rank(l + 1);
         }
@@ -986,7 +1024,7 @@ __global__ void __launch_bounds__(kTopoBlock) topo_write_k(int64_t n, const uint
     if (i == n - 1) {
         for (int l = 0; l <= lam; l++) {
             int c = lvoff[l + 1] - 1;
-            if (c >= cap) { latch_err(st, kErrCells); return; }
+            if (outside(c)) { latch_err(st, kErrCells); return; }
             clink[4 * c + 3] = (int)n;
             if (l < lam) clink[4 * c + 1] = lvoff[l + 2];
         }
@@ -1018,6 +1056,7 @@ struct GroupArgs {
     int64_t cap;
     unsigned *words;   // look-back words, zero before the launch
     int *ticket;
+    LbWait wait;
     int4 *groups;
     int *garrive;
     DevState *st;
@@ -1067,13 +1106,14 @@ __device__ void write_groups(const GroupArgs &A, GroupSmem &S) {
         S.first[threadIdx.x] = lk.z;
         S.end[threadIdx.x] = lk.w;
         if (wid == 0) {
-            if (lane == 0) lb_store(A.words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
+            if (lane == 0 && tile != A.wait.hold)
+                lb_store(A.words + tile, (tile ? kLbSum : kLbPrefix) | (unsigned)total);
             unsigned before = 0;
-            const bool ok = lb_sum_before(A.words, tile, before);
+            const bool ok = lb_sum_before(A.words, tile, A.wait.polls, before);
             if (lane == 0) {
                 if (ok && tile) lb_store(A.words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
                 if (!ok) latch_err(A.st, kErrTimeout);
-                if (ok && c0 + A.tc >= ncell) A.st->ngroup = (int)before + total;
+                lb_total(&A.st->ngroup, ok, c0 + A.tc >= ncell, (int)before + total);
                 S.before = before;
                 S.ok = ok;
             }
@@ -1372,8 +1412,8 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
     topo_count_k<<<nblk, kTopoBlock, win, s>>>(n, skey, c->cfg.n_leaf, w.moff, M, w.dlev, w.lam, w.lvcnt, nblk);
     count_launch(c);
     unsigned *lb = w.lb + kLbScan;   // cleared by bounds_k
-    if ((r = scan_launch(c, w.lvcnt, (int64_t)kLevels * nblk, &w.st->ncell, lb + 1, reinterpret_cast<int *>(lb), s)) !=
-        RV_OK)
+    if ((r = scan_launch(c, w.lvcnt, (int64_t)kLevels * nblk, &w.st->ncell, lb + 1, reinterpret_cast<int *>(lb),
+                         w.lb + kLbGaveUp, s)) != RV_OK)
         return r;
     topo_write_k<<<nblk, kTopoBlock, 0, s>>>(n, skey, w.dlev, w.lam, w.lvcnt, nblk, c->cell_cap, w.moff, M, w.cbox,
                                              w.clink, w.cparent, w.carrive, w.mroot, w.st);
@@ -1383,8 +1423,8 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
     const int gblocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(c->cell_cap, tc), c->num_sms));
     const int mblocks = grid_for(c, c->cell_cap, 256);
     const GroupArgs GA{skey, w.cbox, clink4, w.cparent, c->cfg.group, 16 * c->cfg.group, tc, c->cell_cap,
-                       w.lb + kLbGroups(c->n_max) + 1, reinterpret_cast<int *>(w.lb + kLbGroups(c->n_max)), w.groups,
-                       w.garrive, w.st};
+                       w.lb + kLbGroups(c->n_max) + 1, reinterpret_cast<int *>(w.lb + kLbGroups(c->n_max)),
+                       lb_wait(c, kLbStageGroups), w.groups, w.garrive, w.st};
     const MomentArgs MA{n, w.pos, w.cbox, clink4, w.cparent, w.carrive, w.cmom, c->cell_cap, w.moff, M, w.mbounds, w.st};
     // (one wave of latency-bound blocks as long as the cells fit it)
     if (n < kLatencyBuild) groups_moments_k<8><<<gblocks + mblocks, 256, 0, s>>>(GA, MA, gblocks);

@@ -58,8 +58,10 @@ static SelRule sel_rule(int mode, float radius, const float *m, float gamma) {
     return R;
 }
 
+// (it also clears the total that the scan after it adds up)
 __global__ void sel_radius_flag_k(int64_t n, const float *x, const float *y, const float *z, const float *cdev,
-                                  float4 chost, SelRule R, int *flag) {
+                                  float4 chost, SelRule R, int *flag, int *total) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *total = 0;
     const float3 c = centre_of(cdev, make_float3(chost.x, chost.y, chost.z));
     const float mc = cdev ? cdev[3] : chost.w;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -69,6 +71,11 @@ __global__ void sel_radius_flag_k(int64_t n, const float *x, const float *y, con
 __global__ void sel_radius_write_k(int64_t n, const float *x, const float *y, const float *z, const float *cdev,
                                    float4 chost, SelRule R, const int *ofs, const int *total, int cap, int *idx,
                                    int *count, DevState *st) {
+    const int t = *total;
+    if (t < 0) {   // the scan gave up: no offsets, so nothing is selected
+        if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
+        return;
+    }
     const float3 c = centre_of(cdev, make_float3(chost.x, chost.y, chost.z));
     const float mc = cdev ? cdev[3] : chost.w;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -78,9 +85,7 @@ __global__ void sel_radius_write_k(int64_t n, const float *x, const float *y, co
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int t = *total;
         *count = min(t, cap);
-        st->n_pert = min(t, cap);
         if (t > cap) latch_err(st, kErrPert);
     }
 }
@@ -93,8 +98,9 @@ __global__ void sel_knn_keys_k(int64_t n, const float *x, const float *y, const 
         key[i] = (uint64_t)__float_as_uint(dist2_f32(x[i], y[i], z[i], c.x, c.y, c.z));
 }
 
-__global__ void sel_knn_write_k(const int *sorted_idx, int64_t n, int k, int *idx, int *count, DevState *st) {
-    int kk = (int)min((int64_t)k, n);
+__global__ void sel_knn_write_k(const int *sorted_idx, int64_t n, int k, const unsigned *gave_up, int *idx, int *count,
+                                DevState *st) {
+    int kk = *gave_up ? 0 : (int)min((int64_t)k, n);   // the sort gave up: nothing is selected
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < kk; p += gridDim.x * blockDim.x) idx[p] = sorted_idx[p];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *count = kk;
@@ -326,10 +332,14 @@ static rv_status select_nearest(rv_ctx *c, const SelNear &A, int members, int64_
 
 // Eq. 1 ingredients from the stars sorted by FP32 squared distance (keys =
 // the d2 bits, ties by index): r(<2 M_bh), sigma of the k nearest, M_bh / sigma^2.
-// One thread, sums in distance order in FP64, exactly as the rule reads.
+// One thread, sums in distance order in FP64, exactly as the rule reads. out[3] =
+// 1 if the sort gave up (nothing else is written then).
 __global__ void influence_k(int64_t n, const uint64_t *skey, const int *sidx, const float *vx, const float *vy,
-                            const float *vz, const float *m, double m_bh, int64_t k, double *out) {
+                            const float *vz, const float *m, double m_bh, int64_t k, const unsigned *gave_up,
+                            double *out) {
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    out[3] = *gave_up ? 1.0 : 0.0;
+    if (*gave_up) return;
     double cum = 0.0, r2m = __longlong_as_double(0x7ff0000000000000ll);
     for (int64_t i = 0; i < n; i++) {
         cum = __dadd_rn(cum, (double)m[sidx[i]]);
@@ -373,9 +383,9 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
     if (mode == 1 || mode == 3) {
         const SelRule R = sel_rule(mode, radius, m, gamma);
         if (n == 0) return cuda_check(c, cudaMemsetAsync(count, 0, sizeof(int), s), "select");
-        sel_radius_flag_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, ch, R, w.sel_flag);
+        int *total = &w.st->n_pert;
+        sel_radius_flag_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, ch, R, w.sel_flag, total);
         count_launch(c);
-        int *total = &w.st->n_pert;  // scratch for the total; overwritten by the clamped count
         rv_status r = exclusive_scan(c, w.sel_flag, n, total, s);
         if (r != RV_OK) return r;
         sel_radius_write_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, ch, R, w.sel_flag, total, cap, idx,
@@ -400,7 +410,8 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
         int *si;
         rv_status r = radix_sort(c, n, 4, &sk, &si, s);
         if (r != RV_OK) return r;
-        sel_knn_write_k<<<ceil_div(std::min<int64_t>(k, n), 256), 256, 0, s>>>(si, n, std::min(k, cap), idx, count, w.st);
+        sel_knn_write_k<<<ceil_div(std::min<int64_t>(k, n), 256), 256, 0, s>>>(si, n, std::min(k, cap), w.lb + kLbGaveUp,
+                                                                                      idx, count, w.st);
         count_launch(c);
     }
     return cuda_check(c, cudaGetLastError(), "select perturbers");
@@ -418,11 +429,16 @@ rv_status influence_radius(rv_ctx *c, int64_t n, const float *x, const float *y,
     int *si;
     rv_status r = radix_sort(c, n, 4, &sk, &si, s);
     if (r != RV_OK) return r;
-    influence_k<<<1, 32, 0, s>>>(n, sk, si, vx, vy, vz, m, m_bh, std::min<int64_t>(n_sigma, n), w.out8);
+    influence_k<<<1, 32, 0, s>>>(n, sk, si, vx, vy, vz, m, m_bh, std::min<int64_t>(n_sigma, n),
+                                 w.lb + kLbGaveUp, w.out8);
     count_launch(c);
-    r = cuda_check(c, cudaMemcpyAsync(out, w.out8, 3 * sizeof(double), cudaMemcpyDeviceToHost, s), "influence");
+    double res[4] = {0, 0, 0, 0};
+    r = cuda_check(c, cudaMemcpyAsync(res, w.out8, sizeof res, cudaMemcpyDeviceToHost, s), "influence");
     if (r == RV_OK) r = cuda_check(c, cudaStreamSynchronize(s), "influence");
-    return r;
+    if (r != RV_OK) return r;
+    if (res[3] != 0.0) return set_err(c, RV_E_TIMEOUT, "a wait of the star sort gave up");
+    for (int k = 0; k < 3; k++) out[k] = res[k];
+    return RV_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -447,11 +463,13 @@ __global__ void sel_member_keys_k(const int64_t *moff, int bpm, const float *x, 
 // member m: its first min(k, n_m) sorted slots (k nearest), or its leading
 // "inside" slots (radius), written to idx[m cap ..], count to npert[m]
 __global__ void sel_member_write_k(const int64_t *moff, const uint64_t *skey, const int *sidx, int mode, int k,
-                                   int cap, int C, int j, int *idx, int *npert, DevState *st) {
+                                   int cap, int C, int j, const unsigned *gave_up, int *idx, int *npert, DevState *st) {
     const int m = blockIdx.x;
     const int64_t s = moff[m], e = moff[m + 1];
     int cnt;
-    if (mode == 2) {
+    if (*gave_up) {   // the sort gave up: nothing is selected
+        cnt = 0;
+    } else if (mode == 2) {
         cnt = (int)min((int64_t)k, e - s);
     } else {
         // first "outside" key in the member's slots
@@ -852,7 +870,7 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 if ((r = radix_sort(c, sys->n, sys->pert_mode == 2 ? 4 : 1, &sk, &si, s, true)) != RV_OK)
                     return r;
                 sel_member_write_k<<<M, 256, 0, s>>>(w.moff, sk, si, sys->pert_mode, sys->pert_k, cap, C, j,
-                                                     w.pert_idx, w.npert, w.st);
+                                                     w.lb + kLbGaveUp, w.pert_idx, w.npert, w.st);
                 count_launch(c);
             }
         }

@@ -50,21 +50,25 @@ __device__ __forceinline__ bool absorbed(const DevState *st, float x, float y, f
     return d2 < st->absorb[3];
 }
 
+// (it also clears the total that the scan after it adds up)
 __global__ void absorb_flag_k(int64_t n, const float *x, const float *y, const float *z, const DevState *st,
-                              int *flag) {
+                              int *flag, int *total) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *total = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         flag[i] = absorbed(st, x[i], y[i], z[i]) ? 1 : 0;
 }
 
 __global__ void absorb_write_k(int64_t n, const float *x, const float *y, const float *z, const DevState *st,
                                const int *ofs, const int *total, int cap, int *idx, int *count, double *r_chain) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (absorbed(st, x[i], y[i], z[i])) {
-            const int p = ofs[i];
-            if (p < cap) idx[p] = (int)i;
-        }
+    const int found = n > 0 ? *total : 0;
+    if (found >= 0)   // (-1: the scan gave up, there are no offsets)
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+            if (absorbed(st, x[i], y[i], z[i])) {
+                const int p = ofs[i];
+                if (p < cap) idx[p] = (int)i;
+            }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *count = n > 0 ? *total : 0;
+        *count = max(found, 0);
         if (r_chain) *r_chain = __dsqrt_rn(st->absorb[3]);
     }
 }
@@ -92,7 +96,7 @@ rv_status rv_chain_absorb(rv_ctx *c, int64_t n, const float *x, const float *y, 
     count_launch(c);
     int *total = &w.st->n_pert;   // scratch for the scan's total
     if (n > 0) {
-        absorb_flag_k<<<grid, 256, 0, s>>>(n, x, y, z, w.st, w.sel_flag);
+        absorb_flag_k<<<grid, 256, 0, s>>>(n, x, y, z, w.st, w.sel_flag, total);
         count_launch(c);
         rv_status r = exclusive_scan(c, w.sel_flag, n, total, s);
         if (r != RV_OK) return r;

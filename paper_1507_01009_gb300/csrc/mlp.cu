@@ -1236,8 +1236,8 @@ static rv_status read_ncell(rv_ctx *c, cudaStream_t s, int *ncell, int *ngroup) 
     cudaError_t e = cudaMemcpyAsync(v, &c->w.st->ncell, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_check(c, e, "tree size");
-    *ncell = (int)std::min<int64_t>(v[0], c->cell_cap);
-    *ngroup = v[1];
+    *ncell = (int)std::min<int64_t>(std::max(v[0], 0), c->cell_cap);   // (-1: the build gave up)
+    *ngroup = std::max(v[1], 0);
     return RV_OK;
 }
 

@@ -497,8 +497,8 @@ rv_status rv_get_tree(rv_ctx *c, rv_tree_view *out, void *stream) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_check(c, e, "get tree");
     out->n = c->n;
-    out->ncell = std::min<int64_t>(sz[0], c->cell_cap);
-    out->ngroup = sz[1];
+    out->ncell = std::min<int64_t>(std::max(sz[0], 0), c->cell_cap);   // (-1: the build gave up)
+    out->ngroup = std::max(sz[1], 0);
     out->keys = c->w.skey;
     out->perm = c->w.perm;
     out->pos = reinterpret_cast<const float *>(c->w.pos);
@@ -545,6 +545,15 @@ rv_status rv_sync_status(rv_ctx *c, void *stream) {
         case kErrTimeout: return set_err(c, RV_E_TIMEOUT, "a tensor-core completion wait timed out");
         default: return set_err(c, RV_E_CUDA, "unknown device error %d", err);
     }
+}
+
+rv_status rv_lookback_selftest(rv_ctx *c, int32_t stage, int32_t polls) {
+    if (!c) return RV_E_INVAL;
+    if (stage < 0 || stage > kLbStageGroups || polls < 0 || polls > (1 << 20))
+        return set_err(c, RV_E_INVAL, "need a stage in [0, %d] and 0 <= polls <= 2^20", kLbStageGroups);
+    c->lb_test_stage = stage;
+    c->lb_test_polls = polls;
+    return RV_OK;
 }
 
 int64_t rv_launch_count(const rv_ctx *c) { return c ? (int64_t)c->launches : 0; }

@@ -163,6 +163,7 @@ struct rv_ctx {
     int64_t moff_host[rv::kMaxMembers + 1]; // their star offsets
     int64_t max_member;                     // largest member
     bool moff_on_device;                    // moff_host[0..n_members] already uploaded
+    int lb_test_stage, lb_test_polls;       // rv_lookback_selftest: the stage whose next launch gives up (0: none)
     int pert_members;                       // members whose perturber sets the last force pass chose (0: none)
     // walk timing (rv_profile_walk): event pairs recorded around each walk launch
     bool profile_walk;
@@ -186,6 +187,14 @@ int64_t cell_capacity(int64_t n_max, int n_leaf);
 rv_status set_err(rv_ctx *c, rv_status s, const char *fmt, ...);
 rv_status cuda_check(rv_ctx *c, cudaError_t e, const char *what);
 
+// Bounded look-back waits (build.cu): polls before a wait gives up, and a tile
+// whose words are withheld (-1: none; only the self-test names one).
+struct LbWait {
+    int polls, hold;
+};
+// Stages of rv_lookback_selftest: pass p of a sort is kLbStageSort + p.
+constexpr int kLbStageSort = 1, kLbStageScan = 9, kLbStageGroups = 10;
+
 // build.cu
 rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const float *x, const float *y,
                      const float *z, const float *m, cudaStream_t s);
@@ -193,12 +202,15 @@ rv_status upload_offsets(rv_ctx *c, int M, const int64_t *offsets, cudaStream_t 
 rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, cudaStream_t s,
                      bool member_pass = false, bool counted = false, const float4 *xyzm = nullptr,
                      float4 *pos = nullptr);
-rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s);
+rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s);   // *d_total: see scan_k
 int64_t sort_words(int64_t n_max);   // look-back words of a sort pass, for any n <= n_max
 
 // Layout of Workspace::lb (32-bit words): sort tickets [16], digit counts
 // [kKeyPasses][kSortBins], a scan's ticket and words, the groups' ticket and words.
+// The last ticket word is set by a wait of a sort or of the topology's scan that
+// gave up: the kernels that would use what it leaves unwritten do nothing then.
 constexpr int64_t kLbTickets = 0, kLbHist = 16, kLbScan = kLbHist + kKeyPasses * kSortBins;
+constexpr int kLbGaveUp = 15;
 inline int64_t kLbGroups(int64_t n_max) {   // after the longest scan: n flags, or 22 counts per 256 stars
     return kLbScan + 2 + (n_max + kScanChunk - 1) / kScanChunk + 1;
 }

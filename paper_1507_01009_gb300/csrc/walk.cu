@@ -919,7 +919,7 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
     if (REC && threadIdx.x < kLevels) rec_thr[threadIdx.x] = A.rec.thr[threadIdx.x];
     __syncthreads();
     char *wsm = smem + wib * warp_smem_bytes(A.tile);
-    const int nitem = A.n_extra + (A.order ? A.st->walk.nitem : A.st->ngroup * A.parts);
+    const int nitem = A.n_extra + (A.order ? A.st->walk.nitem : max(A.st->ngroup, 0) * A.parts);
     while (true) {
         int gi = 0;
         if (lane == 0) gi = atomicAdd(&A.st->walk.next_item, 1);

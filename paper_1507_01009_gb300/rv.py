@@ -30,7 +30,7 @@ EXPORTS = ["rv_default_config", "rv_workspace_size", "rv_create", "rv_destroy", 
            "rv_block_start", "rv_block_steps", "rv_block_levels", "rv_block_count", "rv_chain_start_radius", "rv_get_tree", "rv_walk_stats", "rv_sync_status",
            "rv_profile_walk", "rv_walk_time", "rv_launch_count", "rv_last_error", "rv_mlp_param_bytes",
            "rv_mlp_scratch_bytes", "rv_mlp_init", "rv_mlp_forward", "rv_mlp_gradient", "rv_mlp_adam",
-           "rv_mlp_samples", "rv_tree_forces_mlp", "rv_wait_selftest", "rv_mlp_fit_feature_box",
+           "rv_mlp_samples", "rv_tree_forces_mlp", "rv_wait_selftest", "rv_lookback_selftest", "rv_mlp_fit_feature_box",
            "rv_mlp_set_feature_box", "rv_direct_fp64_scratch_bytes", "rv_direct_fp64", "rv_mlp_train_scratch_bytes",
            "rv_mlp_train", "rv_mlp_state_bytes", "rv_mlp_save", "rv_mlp_load", "rv_chain_absorb", "rv_chain_escape"]
 
@@ -147,6 +147,7 @@ def _declare(L):
     L.rv_mlp_samples.argtypes = [vp, f32, f32, i64, C.c_uint64, vp, vp, vp, vp]
     L.rv_tree_forces_mlp.argtypes = [vp, vp, f32, f32, f32, vp, vp, vp, vp, vp, i32, vp, vp, vp]
     L.rv_wait_selftest.argtypes = [i64, i32, vp, vp]
+    L.rv_lookback_selftest.argtypes = [vp, i32, i32]
     L.rv_mlp_fit_feature_box.argtypes = [vp, i64, vp, vp]
     L.rv_mlp_set_feature_box.argtypes = [vp, vp, vp, vp]
     L.rv_direct_fp64_scratch_bytes.argtypes = [i64]
@@ -392,6 +393,10 @@ class Context:
 
     def sync_status(self, stream=None):
         self._check(self.L.rv_sync_status(self.h, _stream(stream)))
+
+    def lookback_selftest(self, stage, polls=0):
+        """rv_lookback_selftest: the next launch of `stage` gives up its look-back waits."""
+        self._check(self.L.rv_lookback_selftest(self.h, int(stage), int(polls)))
 
     # --- chain ---
     def perturber_forces(self, chain_m, chain_x, pert_m, pert_x, stream=None):
