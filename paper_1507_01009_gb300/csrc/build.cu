@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int
         const bool ok = lb_sum_before(words, tile, wait.polls, before);
         if (threadIdx.x == 0) {
             if (ok && tile) lb_store(words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
-            if (!ok) latch_err(st, kErrTimeout);
+            if (!ok) latch_err(st, kErrLookback);
             sbefore = before;
             sok = ok;
             lb_total(d_total, ok, tile == (int)gridDim.x - 1, (int)before + total);
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_k(int64_t n, const uin
     S.gbase[d0 + 1] = first1 + (int)b1 - (ex + tot0);
     if (__syncthreads_or(fail)) {   // a wait gave up: nothing is written
         if (threadIdx.x == 0) {
-            latch_err(st, kErrTimeout);
+            latch_err(st, kErrLookback);
             lb_store(gave_up, 1u);
         }
         return;
@@ -1112,7 +1112,7 @@ __device__ void write_groups(const GroupArgs &A, GroupSmem &S) {
             const bool ok = lb_sum_before(A.words, tile, A.wait.polls, before);
             if (lane == 0) {
                 if (ok && tile) lb_store(A.words + tile, kLbPrefix | ((before + (unsigned)total) & kLbCount));
-                if (!ok) latch_err(A.st, kErrTimeout);
+                if (!ok) latch_err(A.st, kErrLookback);
                 lb_total(&A.st->ngroup, ok, c0 + A.tc >= ncell, (int)before + total);
                 S.before = before;
                 S.ok = ok;

@@ -74,7 +74,7 @@ __host__ __device__ __forceinline__ int parts_of_group(int P, int count) {
 }
 
 // Error codes latched by kernels (first one wins).
-enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kErrPairs = 4, kErrTimeout = 5 };
+enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kErrPairs = 4, kErrTimeout = 5, kErrLookback = 6 };
 
 // Device-resident scalars (one small block in the workspace).
 struct DevState {

@@ -29,6 +29,7 @@ def _gave_up(rvmod, ctx):
     with pytest.raises(rvmod.RvError) as e:
         ctx.sync_status()
     assert e.value.status == rvmod.RV_E_TIMEOUT
+    assert "look-back" in str(e.value)   # not the network's completion wait
 
 
 @pytest.mark.parametrize("members", [1, 3])
