@@ -208,7 +208,19 @@ __device__ __forceinline__ void cube_of(const float lo[3], const float hi[3], do
 // member to finish reduces the blocks' partials (min and max are exact, so the
 // order is free). The first kernel of a build, it also clears the words the
 // later ones count in (zero[nzero]), the member roots and the last build's sizes.
-__global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, const float *x, const float *y,
+//
+// n and the members' number are the launch's own, the offsets are read from the
+// workspace: a caller's graph that is replayed after another build finds that
+// build's offsets there. Then the digit counts would not be those of the n keys
+// that are sorted, so the build is given up (offsets_fit) and no star is read
+// beyond n.
+__device__ __forceinline__ bool offsets_fit(const int64_t *moff, int M, int64_t n) {   // by one block
+    bool bad = threadIdx.x == 0 && (moff[0] != 0 || moff[M] != n);
+    for (int k = threadIdx.x; k < M; k += blockDim.x) bad |= moff[k] > moff[k + 1];
+    return !__syncthreads_or(bad);
+}
+
+__global__ void __launch_bounds__(256) bounds_k(int64_t n, const int64_t *moff, int bpm, const float *x, const float *y,
                                                 const float *z, float *part, int *arrive, double *mbounds,
                                                 DevState *st, unsigned *zero, int64_t nzero, int *mroot) {
     const int m = blockIdx.y;
@@ -219,7 +231,11 @@ __global__ void __launch_bounds__(256) bounds_k(const int64_t *moff, int bpm, co
         mroot[m] = -1;
         if (m == 0) st->ncell = st->ngroup = 0;
     }
-    const int64_t s = moff[m], e = moff[m + 1];
+    if (blockIdx.x == 0 && m == 0 && !offsets_fit(moff, gridDim.y, n) && threadIdx.x == 0) {
+        latch_err(st, kErrOffsets);
+        zero[kLbGaveUp] = 1;   // (after this block's clear of it, above)
+    }
+    const int64_t s = max(moff[m], (int64_t)0), e = min(moff[m + 1], n);
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int64_t i = s + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e; i += (int64_t)bpm * blockDim.x) {
         float v[3] = {x[i], y[i], z[i]};
@@ -391,7 +407,7 @@ __device__ __forceinline__ void count_digits(uint64_t k, int *h) {
 // scattered 4-byte values (each costing a 32-byte sector). The digit counts of
 // all sort passes are taken here, where the keys are in registers (the sort
 // then reads them only to move them), and the first pass's look-back words are cleared.
-__global__ void __launch_bounds__(256) keys_k(const int64_t *moff, int bpm, const float *x, const float *y,
+__global__ void __launch_bounds__(256) keys_k(int64_t n, const int64_t *moff, int bpm, const float *x, const float *y,
                                               const float *z, const float *mass, const double *mbounds, uint64_t *key,
                                               float4 *xyzm, unsigned *ghist, uint4 *words, int64_t nwords4) {
     __shared__ int h[kKeyPasses * kSortBins];
@@ -403,7 +419,7 @@ __global__ void __launch_bounds__(256) keys_k(const int64_t *moff, int bpm, cons
     const double sc = mbounds[5 * m + 4];
     const GridAxis gx = grid_axis(mbounds[5 * m], sc), gy = grid_axis(mbounds[5 * m + 1], sc),
                    gz = grid_axis(mbounds[5 * m + 2], sc);
-    const int64_t s = moff[m], e = moff[m + 1];
+    const int64_t s = max(moff[m], (int64_t)0), e = min(moff[m + 1], n);
     __syncthreads();
     for (int64_t i = s + (int64_t)blockIdx.x * 256 + threadIdx.x; i < e; i += (int64_t)bpm * 256) {
         const float xi = x[i], yi = y[i], zi = z[i];
@@ -700,6 +716,7 @@ constexpr int kSmallThreads = 512, kSmallWarps = kSmallThreads / 32;
 
 struct SmallArgs {
     int n;
+    const int64_t *moff;
     const float *x, *y, *z, *mass;
     double *mbounds;
     int *mroot;
@@ -728,6 +745,10 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_k(SmallArgs A) {
     SmallSmem<ITEMS> &S = *reinterpret_cast<SmallSmem<ITEMS> *>(small_smem);
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5, n = A.n;
     for (int64_t i = t; i < A.nzero; i += kSmallThreads) A.zero[i] = 0;
+    if (!offsets_fit(A.moff, 1, n) && t == 0) {
+        latch_err(A.st, kErrOffsets);
+        A.zero[kLbGaveUp] = 1;
+    }
     // element r of a thread: the warp's consecutive elements in rounds of 32
     const int base = wid * (32 * ITEMS) + lane;
     float px[ITEMS], py[ITEMS], pz[ITEMS];
@@ -1382,16 +1403,16 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
     uint64_t *skey;
     int *perm;
     if (M == 1 && n <= kSmallSort) {
-        skey = w.key_a;
-        perm = w.idx_a;
-        const SmallArgs A{(int)n, x, y, z, m, w.mbounds, w.mroot, w.lb, nzero, skey, perm, w.pos, w.st};
+        skey = w.key_b;   // where the seven passes of a larger system end
+        perm = w.idx_b;
+        const SmallArgs A{(int)n, w.moff, x, y, z, m, w.mbounds, w.mroot, w.lb, nzero, skey, perm, w.pos, w.st};
         static_assert(kSmallSort <= 8 * kSmallThreads, "a thread's share");
         r = n <= 2 * kSmallThreads ? small_sort<2>(c, A, s) : small_sort<8>(c, A, s);
         if (r != RV_OK) return r;
     } else {
         // bounds and keys: blocks per member sized by the largest member
         const int bpm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(big, kBoundsChunk), 512 / M + 1));
-        bounds_k<<<dim3(bpm, M), 256, 0, s>>>(w.moff, bpm, x, y, z, w.bpart, w.barrive, w.mbounds, w.st, w.lb, nzero,
+        bounds_k<<<dim3(bpm, M), 256, 0, s>>>(n, w.moff, bpm, x, y, z, w.bpart, w.barrive, w.mbounds, w.st, w.lb, nzero,
                                               w.mroot);
         count_launch(c);
         // (each block adds its digit counts to the global ones: at least 1024 stars a block)
@@ -1400,7 +1421,7 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
         // groups are written after it (32 B per star of room there, 16 needed)
         float4 *xyzm = reinterpret_cast<float4 *>(w.groups);
         const int64_t tiles = ceil_div(n, kSortThreads * sort_items(n));
-        keys_k<<<dim3(kpm, M), 256, 0, s>>>(w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm, w.lb + kLbHist,
+        keys_k<<<dim3(kpm, M), 256, 0, s>>>(n, w.moff, kpm, x, y, z, m, w.mbounds, w.key_a, xyzm, w.lb + kLbHist,
                                             reinterpret_cast<uint4 *>(w.words[0]), tiles * kSortBins / 4);
         count_launch(c);
         if ((r = radix_sort(c, n, kKeyPasses, &skey, &perm, s, true, true, xyzm, w.pos)) != RV_OK) return r;

@@ -1103,8 +1103,27 @@ rv_status kdk_graph(rv_ctx *c, rv_system *sys, double dt, int nsteps, double *eo
         if (e != cudaSuccess) return cuda_check(c, e, "graph instantiate");
         c->graph = ge;
         c->graph_key = key;
+        c->graph_skey = c->w.skey;
+        c->graph_perm = c->w.perm;
         c->graph_launches = c->launches - l0;
         c->launches = l0;
+    }
+    if (nsteps > 0) {
+        // another build on this context may have come since the capture: the captured kernels
+        // read the member offsets from the workspace, and after the replay the tree in the
+        // workspace is the captured step's
+        const int M = system_members(sys);
+        int64_t tmp[2];
+        const int64_t *off = system_offsets(sys, tmp);
+        rv_status r = upload_offsets(c, M, off, s);
+        if (r != RV_OK) return r;
+        c->n = sys->n;
+        c->max_member = 0;
+        for (int k = 0; k < M; k++) c->max_member = std::max<int64_t>(c->max_member, off[k + 1] - off[k]);
+        c->w.skey = c->graph_skey;
+        c->w.perm = c->graph_perm;
+        c->pert_members = system_chains(sys);
+        c->built = true;
     }
     for (int k = 0; k < nsteps; k++) {
         cudaError_t e = cudaGraphLaunch(c->graph, s);

@@ -544,6 +544,7 @@ rv_status rv_sync_status(rv_ctx *c, void *stream) {
         case kErrPairs: return set_err(c, RV_E_WORKSPACE, "more recorded (group, cell) pairs than the buffer holds");
         case kErrTimeout: return set_err(c, RV_E_TIMEOUT, "a tensor-core completion wait timed out");
         case kErrLookback: return set_err(c, RV_E_TIMEOUT, "a look-back wait of the tree build or of a search gave up; the tree or the selection is empty");
+        case kErrOffsets: return set_err(c, RV_E_INVAL, "a captured build was replayed after another build's member offsets replaced its own; the tree is empty");
         default: return set_err(c, RV_E_CUDA, "unknown device error %d", err);
     }
 }

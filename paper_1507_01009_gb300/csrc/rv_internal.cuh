@@ -74,7 +74,7 @@ __host__ __device__ __forceinline__ int parts_of_group(int P, int count) {
 }
 
 // Error codes latched by kernels (first one wins).
-enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kErrPairs = 4, kErrTimeout = 5, kErrLookback = 6 };
+enum DevErr : int { kErrNone = 0, kErrStack = 1, kErrCells = 2, kErrPert = 3, kErrPairs = 4, kErrTimeout = 5, kErrLookback = 6, kErrOffsets = 7 };
 
 // Device-resident scalars (one small block in the workspace).
 struct DevState {
@@ -175,6 +175,8 @@ struct rv_ctx {
     cudaGraphExec_t graph;
     long long graph_launches;
     unsigned long long graph_key;
+    uint64_t *graph_skey;                   // where the captured build leaves its keys and order
+    int *graph_perm;
     char err[512];
 };
 
@@ -207,8 +209,8 @@ int64_t sort_words(int64_t n_max);   // look-back words of a sort pass, for any 
 
 // Layout of Workspace::lb (32-bit words): sort tickets [16], digit counts
 // [kKeyPasses][kSortBins], a scan's ticket and words, the groups' ticket and words.
-// The last ticket word is set by a wait of a sort or of the topology's scan that
-// gave up: the kernels that would use what it leaves unwritten do nothing then.
+// The last ticket word is set by a wait of a sort that gave up, or by a build whose
+// counts do not fit its stars: the kernels that would use what is then left unwritten do nothing.
 constexpr int64_t kLbTickets = 0, kLbHist = 16, kLbScan = kLbHist + kKeyPasses * kSortBins;
 constexpr int kLbGaveUp = 15;
 inline int64_t kLbGroups(int64_t n_max) {   // after the longest scan: n flags, or 22 counts per 256 stars
