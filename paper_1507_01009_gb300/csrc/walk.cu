@@ -876,7 +876,9 @@ __device__ __forceinline__ bool last_part(int *arrive, int P) {
         if (last) *arrive = 0;
         __threadfence();
     }
-    return __shfl_sync(0xffffffffu, last, 0) != 0;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    __syncwarp();   // the other parts' sums, acquired by lane 0, for every lane (a shuffle orders no memory)
+    return last != 0;
 }
 
 __device__ __forceinline__ float4 part_sum(const Acc &t) {
