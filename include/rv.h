@@ -100,7 +100,9 @@ void rv_destroy(rv_ctx *ctx);
 
 /* Hands librv `bytes` of caller-owned device memory (256-byte aligned), at
  * least rv_workspace_size(). Must stay valid until rv_destroy or the next
- * rv_set_workspace. RV_E_WORKSPACE if too small or misaligned. */
+ * rv_set_workspace. Clears the words that calls expect to find zero and waits
+ * for that; earlier work on this memory on streams that do not synchronise
+ * with the legacy stream must be done. RV_E_WORKSPACE if too small or misaligned. */
 rv_status rv_set_workspace(rv_ctx *ctx, void *dev, size_t bytes);
 
 /* Builds the octree of n stars (device FP32 arrays x, y, z, m; n <= n_max).

@@ -212,6 +212,8 @@ rv_status rv_set_workspace(rv_ctx *c, void *dev, size_t bytes) {
     }
     char *clear = reinterpret_cast<char *>(c->w.selhist), *end = reinterpret_cast<char *>(c->w.st + 1);
     cudaError_t e = cudaMemset(clear, 0, (size_t)(end - clear));
+    // (the first call may come on a stream that does not wait for the legacy one)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     return cuda_check(c, e, "workspace init");
 }
 

@@ -259,6 +259,11 @@ class Context:
         self.ws = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
         base = (self.ws.data_ptr() + 255) & ~255
         self._ws_off = base - self.ws.data_ptr()
+        # the memory's last use may still be under way on this stream, which the clearing of
+        # the workspace (on the legacy stream) does not wait for
+        current = torch.cuda.current_stream()
+        if current.cuda_stream:
+            current.synchronize()
         self._check(self.L.rv_set_workspace(self.h, C.c_void_p(base), nbytes))
         self.n = 0
 

@@ -107,3 +107,41 @@ def test_callers_graph_replayed_after_another_build(rvmod, n, n_other):
     g.replay()
     ctx.sync_status()
     assert all(torch.equal(a, b) for a, b in zip(out, want))
+
+
+def test_workspace_is_clear_before_the_first_call(rvmod):
+    """The words a context expects to find zero are, on whichever stream its first
+    call comes and whatever was queued on the memory before."""
+    import torch
+    n = 20000
+    stars = _stars(n, 10)
+    ref = rvmod.Context(n)
+    ref.build_tree(*stars)
+    want = ref.tree_forces()
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    # the clear waits behind the default stream's work, the build comes on another stream
+    ctx = rvmod.Context(n)
+    torch.cuda._sleep(200_000_000)
+    ctx.ws.fill_(255)
+    ctx._check(ctx.L.rv_set_workspace(ctx.h, ctx.ws.data_ptr() + ctx._ws_off, ctx.ws.numel() - 256))
+    ctx.build_tree(*stars, stream=st)
+    out = [torch.empty(n, device="cuda") for _ in range(4)]
+    st.wait_stream(torch.cuda.current_stream())
+    ctx.n = n
+    ctx.tree_forces(out=out, stream=st)
+    ctx.sync_status(stream=st)
+    assert all(torch.equal(a, b) for a, b in zip(out, want))
+    # the memory's last owner still writes on the context's own stream
+    with torch.cuda.stream(st):
+        old = torch.empty(ctx.ws.numel(), dtype=torch.uint8, device="cuda")
+        at = old.data_ptr()
+        torch.cuda._sleep(200_000_000)
+        old.fill_(255)
+        del old
+        other = rvmod.Context(n)
+        same = other.ws.data_ptr() == at
+        other.build_tree(*stars)
+        got = other.tree_forces()
+        other.sync_status()
+    assert same and all(torch.equal(a, b) for a, b in zip(got, want))
