@@ -74,8 +74,8 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.gorder = (int *)take(4 * (n + 1));
     t.gopart = (uint8_t *)take(n + 1);
     t.garrive = (int *)take(4 * (n + 1));
-    // part sums: P n slots, and P n <= kPartItemsMid group whenever P > 1
-    t.gpartial = (float4 *)take(16 * (size_t)std::min<int64_t>(kMaxParts * n, (int64_t)kPartItemsMid * cfg.group));
+    // part sums and their compensations: P n slots, and P n <= kPartItemsMid group whenever P > 1
+    t.gpartial = (float4 *)take(32 * (size_t)std::min<int64_t>(kMaxParts * n, (int64_t)kPartItemsMid * cfg.group));
     t.gbin = (int *)take(4 * (n + 1));
     t.obins = (int *)take(4 * 1024);
     t.block_count = (unsigned long long *)take(16);

@@ -116,7 +116,7 @@ struct Workspace {
     int *gorder;          // the walk's queue order of the work items: each one's group
     uint8_t *gopart;      // ... and its part of the group's walk
     int *garrive;         // parts of each group's walk that are done
-    float4 *gpartial;     // part sums of the stars of groups walked in several parts [part][sorted star]
+    float4 *gpartial;     // part sums of the stars of groups walked in several parts [part][sums, compensations][sorted star]
     int *gbin;            // each group's cost bin (queue order scratch)
     int *obins;           // bin counts, then next free slots (queue order scratch, 1024)
     unsigned long long *block_count;  // block time steps: active star updates so far

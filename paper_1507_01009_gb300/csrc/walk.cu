@@ -125,7 +125,7 @@ struct WalkArgs {
     float *scost;
     // parts of the groups' walks (Part)
     int parts, n_leaf;
-    float4 *partial;   // [part][sorted star]
+    float4 *partial;   // [part][sums, compensations][sorted star]
     int *garrive;
     // spline softening of the stars (h = 2.8 eps)
     Spline spl;
@@ -881,16 +881,21 @@ __device__ __forceinline__ bool last_part(int *arrive, int P) {
     return last != 0;
 }
 
-__device__ __forceinline__ float4 part_sum(const Acc &t) {
-    return make_float4(t.ax + t.cx, t.ay + t.cy, t.az + t.cz, t.ph + t.cp);
+// A part's sums with their compensations (p: the part's slot of the star, `stride`
+// between the two): a star's total is rounded once, however many parts it has. (The
+// part with the star's own pair is of the size of m / eps, which the end takes out.)
+__device__ __forceinline__ void put_part(float4 *p, int64_t stride, const Acc &t) {
+    p[0] = make_float4(t.ax, t.ay, t.az, t.ph);
+    p[stride] = make_float4(t.cx, t.cy, t.cz, t.cp);
 }
 
-// The parts' sums added in part order (p: the first part's slot, the next ones `stride` apart).
+// The parts' sums added in part order (p: the star's slot of the first part).
 __device__ __forceinline__ Acc add_parts(const float4 *p, int64_t stride, int P) {
     Acc t = {};
     for (int q = 0; q < P; q++) {
-        const float4 v = __ldcg(p + q * stride);
+        const float4 v = __ldcg(p + 2 * q * stride), w = __ldcg(p + (2 * q + 1) * stride);
         nadd(t.ax, t.cx, v.x); nadd(t.ay, t.cy, v.y); nadd(t.az, t.cz, v.z); nadd(t.ph, t.cp, v.w);
+        t.cx += w.x; t.cy += w.y; t.cz += w.z; t.cp += w.w;
     }
     return t;
 }
@@ -1056,7 +1061,7 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
             float4 *slot = A.partial + first;
 #pragma unroll
             for (int h = 0; h < 2; h++)
-                if (lane + 32 * h < s) slot[(int64_t)it.q * A.n + lane + 32 * h] = part_sum(tots[h]);
+                if (lane + 32 * h < s) put_part(slot + (int64_t)2 * it.q * A.n + lane + 32 * h, A.n, tots[h]);
             if (!last_part(A.garrive + it.group, P)) continue;
 #pragma unroll
             for (int h = 0; h < 2; h++)
