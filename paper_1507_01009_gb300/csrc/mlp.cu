@@ -193,11 +193,13 @@ struct GradSmem {
     float red[kGradThreads / 32];
 };
 
-// z -> silu(z) rounded to bfloat16 and silu'(z), from one exponential
+// silu(z) and silu'(z), from one exponential. silu is the quotient itself: as z
+// times the rounded 1 / (1 + e^-z) it takes one rounding more, and more activations
+// fall on the other side of a bfloat16 rounding.
 __device__ __forceinline__ float silu_and_grad(float z, float &grad) {
-    const float s = 1.f / (1.f + expf(-z));
+    const float e = 1.f + expf(-z), s = 1.f / e;
     grad = s * (1.f + z * (1.f - s));
-    return z * s;
+    return z / e;
 }
 
 __global__ void __launch_bounds__(kGradThreads, 1) mlp_grad_k(MlpBlock P, int64_t n, const float *x, const float *tgt,
