@@ -7,6 +7,8 @@
 // centre-of-mass point mass; each member feels the perturbers directly; the
 // centre-of-mass force is corrected by Eq. 3. All of this is unsoftened FP64;
 // sums run in a fixed order so results do not depend on scheduling.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "rv_internal.cuh"
@@ -115,8 +117,8 @@ __global__ void sel_knn_write_k(const int *sorted_idx, int64_t n, int k, const u
 // an octave a bin); (2) the stars up to the bin that holds the k-th are gathered,
 // in any order -- about 1.1 to 1.2 k of them unless many stars lie at nearly
 // one distance; (3) one block a member sorts them. If they do not fit its shared
-// memory it first narrows them digit by digit of the 64-bit (distance, index)
-// value, which is different for every star, so this ends for any input.
+// memory (a centre far outside a compact system sees every star in one bin) the
+// blocks of its cluster first narrow them (near_narrow).
 // Two reads of the positions instead of a four-pass radix sort of all stars:
 // 256 of 2^20 stars 111 -> 30 us of kernels (cold). Members side by side (grid y): a member's
 // candidates go to its own slots of the buffer.
@@ -132,7 +134,9 @@ struct SelNear {
     int C, j;
     float3 chost;
     int k, cap;               // wanted; slots of a member's output
-    int *hist, *ncand;        // [members][kSelBins], [members]: zero before and after
+    int *hist;                // [members][kSelBins]: zero before and after
+    int4 *found;              // [members]: candidates, then the bits set and the bits not set in any key
+                              // of the k-th's bin; zero before and after
     uint64_t *cand, *alt;     // [n] each
     int *idx, *count;         // chain ch's output at idx + ch cap, count + ch (ch = m C + j)
     DevState *st;
@@ -146,20 +150,21 @@ __device__ __forceinline__ float3 near_centre(const SelNear &A, int m) {
     return q ? make_float3(q[0], q[1], q[2]) : A.chost;
 }
 
-// Calls take(key, i) for the block's stars, four of a thread's loaded at once.
+// Calls take(key[4], i[4]) for the block's stars, four of a thread's loaded at once,
+// whole warps together (i < 0: none).
 template <typename F>
 __device__ __forceinline__ void near_scan(const SelNear &A, const float3 &c, int64_t s, int64_t e, F &&take) {
     const int64_t stride = (int64_t)gridDim.x * 256;
-    for (int64_t i = s + (int64_t)blockIdx.x * 256 + threadIdx.x; i < e; i += 4 * stride) {
+    for (int64_t b = s + (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31); b < e; b += 4 * stride) {
         unsigned key[4];
+        int i[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const int64_t q = i + u * stride;
-            if (q < e) key[u] = __float_as_uint(dist2_f32(A.x[q], A.y[q], A.z[q], c.x, c.y, c.z));
+            const int64_t q = b + u * stride + (threadIdx.x & 31), j = min(q, e - 1);
+            i[u] = q < e ? (int)q : -1;
+            key[u] = __float_as_uint(dist2_f32(A.x[j], A.y[j], A.z[j], c.x, c.y, c.z));
         }
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (i + u * stride < e) take(key[u], i + u * stride);
+        take(key, i);
     }
 }
 
@@ -170,7 +175,11 @@ __global__ void __launch_bounds__(256) near_hist_k(SelNear A) {
     const int64_t s = A.moff ? A.moff[m] : 0, e = A.moff ? A.moff[m + 1] : A.n;
     const float3 c = near_centre(A, m);
     __syncthreads();
-    near_scan(A, c, s, e, [&](unsigned key, int64_t) { atomicAdd(&h[near_bin(key)], 1); });
+    near_scan(A, c, s, e, [&](const unsigned *key, const int *i) {
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (i[u] >= 0) atomicAdd(&h[near_bin(key[u])], 1);
+    });
     __syncthreads();
     for (int b = threadIdx.x; b < kSelBins; b += 256)
         if (h[b]) atomicAdd(&A.hist[(int64_t)m * kSelBins + b], h[b]);
@@ -231,59 +240,165 @@ __global__ void __launch_bounds__(256) near_gather_k(SelNear A) {
     int bin, before;
     find_bin<256>(A.hist + (int64_t)m * kSelBins, need, sw, found, bin, before);
     const float3 c = near_centre(A, m);
-    near_scan(A, c, s, e, [&](unsigned key, int64_t i) {
-        if (near_bin(key) <= bin) {
-            const unsigned act = __activemask();
-            const int leader = __ffs(act) - 1;
-            int at = 0;
-            if ((int)(threadIdx.x & 31) == leader) at = atomicAdd(&A.ncand[m], __popc(act));
-            at = __shfl_sync(act, at, leader) + __popc(act & lanemask_lt());
-            A.cand[s + at] = ((uint64_t)key << 32) | (unsigned)i;
+    unsigned ones = 0, zeros = 0;
+    near_scan(A, c, s, e, [&](const unsigned *key, const int *i) {
+        bool mine[4], any = false;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            mine[u] = i[u] >= 0 && near_bin(key[u]) <= bin;
+            any |= mine[u];
+        }
+        if (!__any_sync(0xffffffffu, any)) return;
+        unsigned in[4];
+        int all = 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            in[u] = __ballot_sync(0xffffffffu, mine[u]);
+            all += __popc(in[u]);
+        }
+        int at = 0;   // (one place in the list for a warp's four rounds: many candidates queue at one counter)
+        if ((threadIdx.x & 31) == 0) at = atomicAdd(&A.found[m].x, all);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (mine[u]) {
+                A.cand[s + at + __popc(in[u] & lanemask_lt())] = ((uint64_t)key[u] << 32) | (unsigned)i[u];
+                if (near_bin(key[u]) == bin) {
+                    ones |= key[u];
+                    zeros |= ~key[u];
+                }
+            }
+            at += __popc(in[u]);
         }
     });
+    ones = __reduce_or_sync(0xffffffffu, ones);
+    zeros = __reduce_or_sync(0xffffffffu, zeros);
+    if ((threadIdx.x & 31) == 0 && (ones | zeros)) {
+        atomicOr(reinterpret_cast<unsigned *>(&A.found[m].y), ones);
+        atomicOr(reinterpret_cast<unsigned *>(&A.found[m].z), zeros);
+    }
 }
 
+// Calls take(ok, value) for this block's share of a candidate list, 32 or 64 KB of it
+// loaded at once (a block's reads are bound by their latency), whole warps together.
+template <int NT, typename F>
+__device__ __forceinline__ void near_share(const uint64_t *a, int rem, int rank, int CL, F &&take) {
+    constexpr int U = NT <= 256 ? 16 : 8;
+    const int lane = threadIdx.x & 31, stride = NT * CL;
+    for (int b = rank * NT + (threadIdx.x & ~31); b < rem; b += U * stride) {
+        unsigned long long w[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (b + u * stride + lane < rem)   // (the list of a later round was written by other blocks: from L2)
+                w[u] = __ldcg(reinterpret_cast<const unsigned long long *>(a) + b + u * stride + lane);
+#pragma unroll
+        for (int u = 0; u < U; u++) take(b + u * stride + lane < rem, (uint64_t)w[u]);
+    }
+}
+
+struct NearSmem {
+    int h[kSelBins], sw[32], found[2], nacc, nrem;
+};
+
+// Narrows `rem` candidates (list a) to what a block sorts, digit by digit of the
+// 64-bit (distance, index) value, which is different for every star, so this
+// ends for any input: what lies below the digit of the k-th goes to the first
+// block's array v (fewer than `want` in all), what shares it to the other list.
+// The CL blocks of a member's cluster share the lists; the counts and v are the
+// first block's. On return v holds acc values and list a the other rem. shift: the
+// first digit's.
 template <int NT>
-__global__ void __launch_bounds__(NT) near_sort_k(SelNear A) {
+__device__ void near_narrow(NearSmem &S, int shift, uint64_t *v, uint64_t *&a, uint64_t *o, int want, int rank,
+                            int CL, int &acc, int &rem) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x;
+    int *h0 = cl.map_shared_rank(S.h, 0), *nacc0 = cl.map_shared_rank(&S.nacc, 0),
+        *nrem0 = cl.map_shared_rank(&S.nrem, 0);
+    uint64_t *v0 = cl.map_shared_rank(v, 0);
+    // the next places of the set lanes at a counter of the first block
+    auto slots = [](int *counter, unsigned set) -> int {
+        int at = 0;
+        if ((threadIdx.x & 31) == 0) at = atomicAdd(counter, __popc(set));
+        return __shfl_sync(0xffffffffu, at, 0) + __popc(set & lanemask_lt());
+    };
+    if (t == 0) S.nacc = 0;
+    for (; acc + rem > kSelCap; shift = max(shift - 11, 0)) {
+        auto digit = [&](uint64_t w) -> int { return (int)(w >> shift) & (kSelBins - 1); };
+        for (int b = t; b < kSelBins; b += NT) S.h[b] = 0;
+        cl.sync();
+        if (t == 0) S.nrem = 0;
+        near_share<NT>(a, rem, rank, CL, [&](bool ok, uint64_t w) {
+            if (ok) atomicAdd(&S.h[digit(w)], 1);
+        });
+        __syncthreads();
+        if (rank != 0)
+            for (int b = t; b < kSelBins; b += NT)
+                if (S.h[b]) atomicAdd(h0 + b, S.h[b]);
+        cl.sync();
+        if (rank != 0)
+            for (int b = t; b < kSelBins; b += NT) S.h[b] = h0[b];
+        __syncthreads();
+        int bin, before;
+        find_bin<NT>(S.h, want - acc, S.sw, S.found, bin, before);
+        if (S.h[bin] != rem) {   // (all share the digit: nothing to move)
+            near_share<NT>(a, rem, rank, CL, [&](bool ok, uint64_t w) {
+                const int d = ok ? digit(w) : kSelBins;
+                const unsigned below = __ballot_sync(0xffffffffu, d < bin), same = __ballot_sync(0xffffffffu, d == bin);
+                if (below) {
+                    const int at = slots(nacc0, below);
+                    if (d < bin) v0[at] = w;
+                }
+                if (same) {
+                    const int at = slots(nrem0, same);
+                    if (d == bin) o[at] = w;
+                }
+            });
+            cl.sync();
+            acc = *nacc0;
+            rem = *nrem0;
+            uint64_t *q = a;
+            a = o;
+            o = q;
+        }
+        cl.sync();   // the first block's counts are read before it goes on
+    }
+}
+
+// Grid: CL blocks a member (a cluster); the first one sorts, the others only
+// help to narrow.
+template <int NT>
+__global__ void __launch_bounds__(NT) near_sort_k(SelNear A, int CL) {
     extern __shared__ __align__(16) char near_smem[];
     uint64_t *v = reinterpret_cast<uint64_t *>(near_smem);   // [kSelCap]
-    __shared__ int h[kSelBins], sw[32], found[2], nacc, nrem;
-    const int m = blockIdx.x, t = threadIdx.x;
+    __shared__ NearSmem S;
+    const int m = blockIdx.x / CL, rank = blockIdx.x % CL, t = threadIdx.x;
     const int64_t s = A.moff ? A.moff[m] : 0, e = A.moff ? A.moff[m + 1] : A.n;
     const int64_t ch = (int64_t)m * A.C + A.j;
     int *hist = A.hist + (int64_t)m * kSelBins;
     const int take = (int)min((int64_t)A.k, e - s);
-    int rem = take > 0 ? A.ncand[m] : 0, acc = 0;
+    // (few candidates: the first block may clear the count before the others read it, and
+    // they end either way; many: it is cleared after the cluster has met)
+    int rem = take > 0 ? *(volatile int *)&A.found[m].x : 0, acc = 0;
+    if (rank != 0 && rem <= kSelCap) return;
     __syncthreads();
-    for (int b = t; b < kSelBins; b += NT) hist[b] = 0;   // ready for the next selection
-    if (t == 0) {
-        A.ncand[m] = 0;
-        nacc = 0;
-    }
-    uint64_t *a = A.cand + s, *o = A.alt + s;
-    for (int shift = 53; acc + rem > kSelCap; shift = max(shift - 11, 0)) {
-        for (int b = t; b < kSelBins; b += NT) h[b] = 0;
-        if (t == 0) nrem = 0;
-        __syncthreads();
-        for (int i = t; i < rem; i += NT) atomicAdd(&h[(int)(a[i] >> shift) & (kSelBins - 1)], 1);
-        __syncthreads();
-        int bin, before;
-        find_bin<NT>(h, take - acc, sw, found, bin, before);
-        for (int i = t; i < rem; i += NT) {
-            const uint64_t w = a[i];
-            const int d = (int)(w >> shift) & (kSelBins - 1);
-            if (d < bin) v[atomicAdd(&nacc, 1)] = w;          // among the k nearest: at most take of these
-            else if (d == bin) o[atomicAdd(&nrem, 1)] = w;
+    uint64_t *a = A.cand + s;
+    if (rem > kSelCap) {
+        // all candidates in the k-th's bin: they share its bits (the last bin holds several values),
+        // and the first digit starts at the highest bit in which any two differ
+        int bin, before, shift = 53;
+        find_bin<NT>(hist, take, S.sw, S.found, bin, before);
+        if (before == 0 && bin < kSelBins - 1) {
+            const unsigned differ = (unsigned)A.found[m].y & (unsigned)A.found[m].z;
+            const int top = differ ? 63 - __clz(differ) : 31 - __clz((int)(e - 1));
+            shift = max(top - 10, 0);
         }
-        __syncthreads();
-        acc = nacc;
-        rem = nrem;
-        uint64_t *q = a;
-        a = o;
-        o = q;
-        __syncthreads();
+        near_narrow<NT>(S, shift, v, a, A.alt + s, take, rank, CL, acc, rem);
     }
-    for (int i = t; i < rem; i += NT) v[acc + i] = a[i];
+    if (rank != 0) return;
+    for (int b = t; b < kSelBins; b += NT) hist[b] = 0;   // ready for the next selection
+    if (t == 0) A.found[m] = make_int4(0, 0, 0, 0);
+    for (int i = t; i < rem; i += NT) v[acc + i] = __ldcg(reinterpret_cast<const unsigned long long *>(a) + i);
     int size = 2;
     while (size < acc + rem) size <<= 1;
     for (int i = acc + rem + t; i < size; i += NT) v[i] = ~0ull;
@@ -313,21 +428,49 @@ __global__ void __launch_bounds__(NT) near_sort_k(SelNear A) {
     }
 }
 
-static rv_status select_nearest(rv_ctx *c, const SelNear &A, int members, int64_t largest, cudaStream_t s) {
+// Blocks of a cluster that narrow a member's candidates together: one block reads
+// them at the rate of its latency (25 GB/s). us a search of 256, 4000 of 2^20 stars
+// from 1000 and 10^6 radii away, one block | eight | a sort of all stars: 57, 740
+// and 2280, 720 | 60, 124 and 126, 106 | 156 and 144. From inside the system, where a block's
+// memory holds the candidates, nothing changes (27 us; the other blocks end at
+// once). A block alone does for systems of up to 2^14 stars (from outside 85 to 95 us
+// of 5000), and in an ensemble, whose blocks are many, for members of up to 2^16.
+constexpr int kSelBlocks = 8;
+static int near_blocks(int members, int64_t largest, int sms) {
+    return largest > (members == 1 ? 1 << 14 : 1 << 16) && members * kSelBlocks <= 2 * sms ? kSelBlocks : 1;
+}
+
+template <int NT>
+static cudaError_t near_sort(const SelNear &A, int members, int CL, cudaStream_t s) {
     const size_t smem = sizeof(uint64_t) * kSelCap;
+    cudaError_t e = cudaFuncSetAttribute(near_sort_k<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(members * CL);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, near_sort_k<NT>, A, CL);
+}
+
+static rv_status select_nearest(rv_ctx *c, const SelNear &A, int members, int64_t largest, cudaStream_t s) {
     // (few candidates: a small block, whose barriers are cheaper)
     const bool few = std::min(A.k, A.cap) <= 512;
-    cudaError_t e = few ? cudaFuncSetAttribute(near_sort_k<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                        : cudaFuncSetAttribute(near_sort_k<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_check(c, e, "select nearest");
+    const int CL = near_blocks(members, largest, c->num_sms);
     // about 1024 stars a block, four blocks an SM over all members
     const int bx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(largest, 1024), (int64_t)c->num_sms * 4 / members + 1));
     near_hist_k<<<dim3(bx, members), 256, 0, s>>>(A);
     near_gather_k<<<dim3(bx, members), 256, 0, s>>>(A);
-    if (few) near_sort_k<256><<<members, 256, smem, s>>>(A);
-    else near_sort_k<1024><<<members, 1024, smem, s>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = few ? near_sort<256>(A, members, CL, s) : near_sort<1024>(A, members, CL, s);
     c->launches += 3;
-    return cuda_check(c, cudaGetLastError(), "select nearest");
+    return cuda_check(c, e, "select nearest");
 }
 
 // Eq. 1 ingredients from the stars sorted by FP32 squared distance (keys =
@@ -401,7 +544,7 @@ rv_status select_perturbers(rv_ctx *c, int64_t n, const float *x, const float *y
         if (std::min<int64_t>(k, n) <= kSelMaxK) {
             // (one member: an output shorter than k is simply the nearest cap of them)
             const SelNear A{nullptr, n, x, y, z, centre_dev, 1, 0, make_float3(ch.x, ch.y, ch.z), std::min(k, cap), cap,
-                            w.selhist, w.selcand, w.key_a, w.key_b, idx, count, w.st, true};
+                            w.selhist, w.selfound, w.key_a, w.key_b, idx, count, w.st, true};
             if (A.k > 0) return select_nearest(c, A, 1, n, s);
         }
         sel_knn_keys_k<<<grid_n(c, n), 256, 0, s>>>(n, x, y, z, centre_dev, make_float3(ch.x, ch.y, ch.z), w.key_a);
@@ -853,7 +996,7 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 // the sort buffers are shared with the tree build, which comes next
                 if (sys->pert_mode == 2 && sys->pert_k > 0) {
                     const SelNear A{w.moff, sys->n, sys->x, sys->y, sys->z, w.extra_xyzm, C, j, make_float3(0.f, 0.f, 0.f),
-                                    sys->pert_k, cap, w.selhist, w.selcand, w.key_a, w.key_b, w.pert_idx, w.npert, w.st,
+                                    sys->pert_k, cap, w.selhist, w.selfound, w.key_a, w.key_b, w.pert_idx, w.npert, w.st,
                                     false};
                     int64_t big = 1;
                     for (int k = 0; k < M; k++) big = std::max<int64_t>(big, off[k + 1] - off[k]);

@@ -103,7 +103,7 @@ size_t layout(int64_t n_max, const rv_config &cfg, char *base, Workspace *w, int
     t.gstack = (int *)take(4 * (size_t)kStackSpillWarps * kStackSpill);
     // zero when the workspace is set, kept so by what uses them: side by side, one clear
     t.selhist = (int *)take(4 * (size_t)kMaxMembers * kSelBins);
-    t.selcand = (int *)take(4 * kMaxMembers);
+    t.selfound = (int4 *)take(16 * kMaxMembers);
     t.barrive = (int *)take(4 * kMaxMembers);
     t.st = (DevState *)take(sizeof(DevState));
     if (w) *w = t;

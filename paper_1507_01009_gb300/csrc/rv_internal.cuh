@@ -132,7 +132,7 @@ struct Workspace {
     double *red;          // energy partial sums
     int *sel_flag;        // perturber selection flags (n)
     int *selhist;         // nearest selection: distance counts per member [kMaxMembers][kSelBins], 0 between calls
-    int *selcand;         // ... and candidates gathered [kMaxMembers], 0 between calls
+    int4 *selfound;       // ... and what was gathered [kMaxMembers], 0 between calls
     // members (independent systems sharing one build and one walk)
     int64_t *moff;        // member star offsets [kMaxMembers + 1]
     double *mbounds;      // per member: min x, y, z, L, 2^21 / L

@@ -1,0 +1,98 @@
+"""k nearest stars seen from far outside the system, where (nearly) every star
+lies in one bin of the distances' leading bits: the narrowing before the sort,
+by one block and by a cluster of blocks (more than 16384 stars)."""
+import numpy as np
+import pytest
+
+from gpu_helpers import hernquist32
+
+pytestmark = pytest.mark.gpu
+
+
+def _nearest(p, centre, k):
+    """FP32 squared distances, one rounding per operation; ties by index."""
+    import torch
+    d = p - torch.tensor(centre, dtype=torch.float32, device="cuda")[:, None]
+    d2 = (d[0] * d[0] + d[1] * d[1]) + d[2] * d[2]
+    return torch.sort(d2, stable=True).indices[:k].int()
+
+
+@pytest.mark.parametrize("k", [1, 256, 513, 5000])
+@pytest.mark.parametrize("n", [8193, 16384, 16385, 300001])
+def test_nearest_from_outside(n, k):
+    """Centres 50, 1000, 10^6 radii away (at the last one the distances are a few FP32
+    values, nearly all ties), coincident stars, and stars with infinite and
+    undefined distances among them."""
+    import torch
+    from paper_1507_01009_gb300 import rv
+    p = torch.from_numpy(hernquist32(n, 17)[0]).cuda().contiguous()
+    far = p.clone()
+    far[0, 5::7] = 3e38
+    far[1, 3::11] = float("nan")
+    ctx = rv.Context(n)
+    for stars, centre in ((p, (50.0, 0, 0)), (p, (0, -1000.0, 3.0)), (p, (1e6, 1e6, 0)), (torch.zeros_like(p), (1.0, 2.0, 3.0)),
+                          (far, (1000.0, 0, 0)), (p, (0, 0, 0))):
+        for _ in range(2):   # the second search starts from the first one's counters
+            idx, count = ctx.select_perturbers(*stars, centre, 2, k=k)
+            kk = min(k, n)
+            assert int(count) == kk
+            assert torch.equal(idx[:kk], _nearest(stars, centre, kk))
+    ctx.sync_status()
+
+
+def test_members_seen_from_outside():
+    """Chains 1000 radii from their members' stars, members on both sides of 65536 stars (a
+    cluster of blocks a member) and empty and small ones: the pull of the selected
+    stars equals that of the stars numpy selects."""
+    import torch
+    from paper_1507_01009_gb300 import rv
+    k = 300
+    for sizes in ([70000, 0, 30000, 40], [9000, 20000]):
+        parts = [hernquist32(n, 40 + n % 7) if n else None for n in sizes]
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        p32 = np.concatenate([p[0] for p in parts if p], axis=1)
+        m32 = np.concatenate([p[1] for p in parts if p])
+        M = len(sizes)
+        at = np.array([[1000.0 * (-1) ** j, 50.0 * j, 0.0] for j in range(M)])
+        S = rv.System(p32, np.zeros_like(p32), m32, chain_m=np.full(M, 0.01), chain_x=at, chain_v=np.zeros((M, 3)),
+                      pert_mode=2, pert_k=k, member_offsets=off)
+        ctx = rv.Context(int(off[-1]))
+        for _ in range(2):
+            ctx.system_forces(S)
+            a, _ = ctx.chain_perturber_forces(S, 0.0, S.chain_x)
+        ctx.sync_status()
+        for j in range(M):
+            p, m = p32[:, off[j]:off[j + 1]], m32[off[j]:off[j + 1]].astype(np.float64)
+            d = p - at[j].astype(np.float32)[:, None]
+            d2 = (d[0] * d[0] + d[1] * d[1]) + d[2] * d[2]
+            i = np.argsort(d2, kind="stable")[:k]
+            r = p[:, i].astype(np.float64) - at[j][:, None]
+            want = (m[i] * r / np.linalg.norm(r, axis=0) ** 3).sum(1)
+            np.testing.assert_allclose(a.cpu().numpy()[3 * j:3 * j + 3], want, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("centre,k", [(1000.0, 4000), (1e6, 256)])
+def test_search_from_outside_is_no_slower_than_a_sort(centre, k):
+    """2^20 stars: the selection against the sort of all stars that longer lists take
+    (more than 5000), the same call and centre."""
+    import torch
+    from paper_1507_01009_gb300 import rv
+    n = 1 << 20
+    p = torch.from_numpy(hernquist32(n, 18)[0]).cuda().contiguous()
+    ctx = rv.Context(n)
+
+    def best(k):
+        t = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            for _ in range(3):
+                ctx.select_perturbers(*p, (centre, 0, 0), 2, k=k, cap=k)
+            a.record()
+            for _ in range(10):
+                ctx.select_perturbers(*p, (centre, 0, 0), 2, k=k, cap=k)
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    assert best(k) <= 1.3 * best(6000)
