@@ -1396,10 +1396,14 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
         return r;
     }
     const int nblk = ceil_div(n, kTopoBlock);
+    // what the build clears and launches follows its own stars, not the context's: cells of n
+    // stars (at most 8 children of every split cell, of which a level has n / (n_leaf + 1))
+    const int64_t cells = std::min<int64_t>(
+        c->cell_cap, M + 2 + kMaxLevel * std::min<int64_t>(n, 8 * n / (c->cfg.n_leaf + 1) + 8));
     // cells a tile of the groups pass (few in small builds: more blocks); cleared
     // first: tickets, digit counts, the look-back words of the topology scan and of that pass
     const int tc = n < (1 << 19) ? 64 : 256;
-    const int64_t nzero = kLbGroups(c->n_max) + 2 + ceil_div(c->cell_cap, tc);
+    const int64_t lb_groups = kLbGroups(n), nzero = lb_groups + 2 + ceil_div(cells, tc);
     uint64_t *skey;
     int *perm;
     if (M == 1 && n <= kSmallSort) {
@@ -1441,10 +1445,10 @@ rv_status build_tree(rv_ctx *c, int n_members, const int64_t *offsets, const flo
     count_launch(c);
     // groups and multipoles
     const int4 *clink4 = reinterpret_cast<const int4 *>(w.clink);
-    const int gblocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(c->cell_cap, tc), c->num_sms));
-    const int mblocks = grid_for(c, c->cell_cap, 256);
+    const int gblocks = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(cells, tc), c->num_sms));
+    const int mblocks = grid_for(c, cells, 256);
     const GroupArgs GA{skey, w.cbox, clink4, w.cparent, c->cfg.group, 16 * c->cfg.group, tc, c->cell_cap,
-                       w.lb + kLbGroups(c->n_max) + 1, reinterpret_cast<int *>(w.lb + kLbGroups(c->n_max)),
+                       w.lb + lb_groups + 1, reinterpret_cast<int *>(w.lb + lb_groups),
                        lb_wait(c, kLbStageGroups), w.groups, w.garrive, w.st};
     const MomentArgs MA{n, w.pos, w.cbox, clink4, w.cparent, w.carrive, w.cmom, c->cell_cap, w.moff, M, w.mbounds, w.st};
     // (one wave of latency-bound blocks as long as the cells fit it)

@@ -213,8 +213,8 @@ int64_t sort_words(int64_t n_max);   // look-back words of a sort pass, for any 
 // counts do not fit its stars: the kernels that would use what is then left unwritten do nothing.
 constexpr int64_t kLbTickets = 0, kLbHist = 16, kLbScan = kLbHist + kKeyPasses * kSortBins;
 constexpr int kLbGaveUp = 15;
-inline int64_t kLbGroups(int64_t n_max) {   // after the longest scan: n flags, or 22 counts per 256 stars
-    return kLbScan + 2 + (n_max + kScanChunk - 1) / kScanChunk + 1;
+inline int64_t kLbGroups(int64_t n) {   // after the longest scan of n stars: n flags, or 22 counts per 256 stars
+    return kLbScan + 2 + (n + kScanChunk - 1) / kScanChunk + 1;
 }
 
 // Opening test on integer grid distances: accept iff d^2 >= thr[level].
