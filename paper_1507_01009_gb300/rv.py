@@ -181,22 +181,25 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
-_CURRENT = None   # (current device, its current stream's handle), bound on first use
+_CURRENT = None   # the handle of torch's current stream, a function bound on first use
 
 
 def _stream(stream=None):
     """The stream's handle (torch's current one by default). torch.cuda.current_stream()
     resolves the device in Python and builds a Stream object, 12 us of a 25 us call;
-    the two calls below give the same handle in under one."""
+    torch's own two calls under it give the same handle in under one, and it is the
+    way back where they are missing (they are not part of torch's public interface)."""
     global _CURRENT
     if stream is not None:
         return stream.cuda_stream
     if _CURRENT is None:
         import torch
         torch.cuda.init()
-        _CURRENT = (torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
-    device, raw = _CURRENT
-    return raw(device())
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _CURRENT = ((lambda: raw(device())) if device and raw else
+                    (lambda: torch.cuda.current_stream().cuda_stream))
+    return _CURRENT()
 
 
 def default_config(**kw) -> rv_config:
