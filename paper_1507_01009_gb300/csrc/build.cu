@@ -100,10 +100,9 @@ __device__ __forceinline__ void lb_total(int *d_total, bool ok, bool last, int t
     else if (last) atomicCAS(d_total, 0, total);
 }
 
-// Exclusive scan of int32 (in place), length *d_len (<= nmax) or nmax; the
-// total to *d_total (lb_total). words, ticket: zero before the launch. gave_up
+// Exclusive scan of n int32 in place; the total to *d_total (lb_total). words, ticket: zero before the launch. gave_up
 // (optional): set if the data is not there, and then nothing is done.
-__global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int *d_len, unsigned *words, int *ticket,
+__global__ void __launch_bounds__(256) scan_k(int *data, int64_t len, unsigned *words, int *ticket,
                                               const unsigned *gave_up, LbWait wait, int *d_total, DevState *st) {
     __shared__ int sw[8], stile;
     __shared__ unsigned sbefore;
@@ -115,7 +114,6 @@ __global__ void __launch_bounds__(256) scan_k(int *data, int64_t nmax, const int
     __syncthreads();
     const int tile = stile;
     if (tile < 0) return;
-    const int64_t len = d_len ? min((int64_t)*d_len, nmax) : nmax;
     const int64_t base = (int64_t)tile * kScanChunk + threadIdx.x * 8;
     int v[8], s = 0;
     if (base + 8 <= len) {   // the tile's start is 32-byte aligned
@@ -168,23 +166,23 @@ static LbWait lb_wait(rv_ctx *c, int stage) {
     return LbWait{c->lb_test_polls, 0};
 }
 
-static rv_status scan_launch(rv_ctx *c, int *data, int64_t nmax, int *d_total, unsigned *words, int *ticket,
+static rv_status scan_launch(rv_ctx *c, int *data, int64_t n, int *d_total, unsigned *words, int *ticket,
                              const unsigned *gave_up, cudaStream_t s) {
-    scan_k<<<ceil_div(nmax, kScanChunk), 256, 0, s>>>(data, nmax, nullptr, words, ticket, gave_up,
-                                                      lb_wait(c, kLbStageScan), d_total, c->w.st);
+    scan_k<<<ceil_div(n, kScanChunk), 256, 0, s>>>(data, n, words, ticket, gave_up, lb_wait(c, kLbStageScan), d_total,
+                                                   c->w.st);
     count_launch(c);
     return cuda_check(c, cudaGetLastError(), "scan");
 }
 
 // *d_total is 0 before; -1 after it means that a wait gave up.
-rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s) {
-    if (nmax <= 0) return RV_OK;
+rv_status exclusive_scan(rv_ctx *c, int *data, int64_t n, int *d_total, cudaStream_t s) {
+    if (n <= 0) return RV_OK;
     // ticket and words side by side: one clear
     unsigned *z = c->w.lb + kLbScan;
-    rv_status r = cuda_check(c, cudaMemsetAsync(z, 0, sizeof(unsigned) * (1 + (size_t)ceil_div(nmax, kScanChunk)), s),
+    rv_status r = cuda_check(c, cudaMemsetAsync(z, 0, sizeof(unsigned) * (1 + (size_t)ceil_div(n, kScanChunk)), s),
                              "scan");
     if (r != RV_OK) return r;
-    return scan_launch(c, data, nmax, d_total, z + 1, reinterpret_cast<int *>(z), nullptr, s);
+    return scan_launch(c, data, n, d_total, z + 1, reinterpret_cast<int *>(z), nullptr, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -585,11 +585,10 @@ rv_status influence_radius(rv_ctx *c, int64_t n, const float *x, const float *y,
 }
 
 // ---------------------------------------------------------------------------
-// perturber selection per member (systems of several members): one stable
-// sort of (member, key) over all stars; member m's stars occupy the same
-// slots [moff[m], moff[m+1]) in sorted order, best first.
-//   k nearest: key = FP32 squared distance bits to the member's centre
-//   radius:    key = 0 inside, 1 outside (inside stars first, ascending index)
+// radius or tidal search per member (systems of several members): one stable
+// sort of (member, key) over all stars, key = 0 inside, 1 outside; member m's stars
+// occupy the same slots [moff[m], moff[m+1]) in sorted order, inside ones first
+// in ascending index.
 // ---------------------------------------------------------------------------
 __global__ void sel_member_keys_k(const int64_t *moff, int bpm, const float *x, const float *y, const float *z,
                                   const float *xyzm, int C, int j, SelRule R, uint64_t *key) {
@@ -599,22 +598,16 @@ __global__ void sel_member_keys_k(const int64_t *moff, int bpm, const float *x, 
     for (int64_t i = moff[m] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < moff[m + 1];
          i += (int64_t)bpm * blockDim.x) {
         float d2 = dist2_f32(x[i], y[i], z[i], cx, cy, cz);
-        key[i] = (R.mode == 2) ? (uint64_t)__float_as_uint(d2) : (sel_inside(R, d2, i, mc) ? 0ull : 1ull);
+        key[i] = sel_inside(R, d2, i, mc) ? 0ull : 1ull;
     }
 }
 
-// member m: its first min(k, n_m) sorted slots (k nearest), or its leading
-// "inside" slots (radius), written to idx[m cap ..], count to npert[m]
-__global__ void sel_member_write_k(const int64_t *moff, const uint64_t *skey, const int *sidx, int mode, int k,
-                                   int cap, int C, int j, const unsigned *gave_up, int *idx, int *npert, DevState *st) {
+// member m: its leading "inside" slots, written to idx[m cap ..], count to npert[m]
+__global__ void sel_member_write_k(const int64_t *moff, const uint64_t *skey, const int *sidx, int cap, int C, int j, const unsigned *gave_up, int *idx, int *npert, DevState *st) {
     const int m = blockIdx.x;
     const int64_t s = moff[m], e = moff[m + 1];
-    int cnt;
-    if (*gave_up) {   // the sort gave up: nothing is selected
-        cnt = 0;
-    } else if (mode == 2) {
-        cnt = (int)min((int64_t)k, e - s);
-    } else {
+    int cnt = 0;
+    if (!*gave_up) {   // (a sort that gave up: nothing is selected)
         // first "outside" key in the member's slots
         int64_t lo = s, hi = e;
         while (lo < hi) {
@@ -994,7 +987,12 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 if (r != RV_OK) return r;
             } else {
                 // the sort buffers are shared with the tree build, which comes next
-                if (sys->pert_mode == 2 && sys->pert_k > 0) {
+                if (sys->pert_mode == 2) {
+                    if (sys->pert_k <= 0) {   // (every chain's count at once)
+                        r = cuda_check(c, cudaMemsetAsync(w.npert, 0, sizeof(int) * NC, s), "select nearest");
+                        if (r != RV_OK) return r;
+                        continue;
+                    }
                     const SelNear A{w.moff, sys->n, sys->x, sys->y, sys->z, w.extra_xyzm, C, j, make_float3(0.f, 0.f, 0.f),
                                     sys->pert_k, cap, w.selhist, w.selfound, w.key_a, w.key_b, w.pert_idx, w.npert, w.st,
                                     false};
@@ -1010,10 +1008,9 @@ rv_status system_forces(rv_ctx *c, rv_system *sys, cudaStream_t s, const BlockSe
                 count_launch(c);
                 uint64_t *sk;
                 int *si;
-                if ((r = radix_sort(c, sys->n, sys->pert_mode == 2 ? 4 : 1, &sk, &si, s, true)) != RV_OK)
-                    return r;
-                sel_member_write_k<<<M, 256, 0, s>>>(w.moff, sk, si, sys->pert_mode, sys->pert_k, cap, C, j,
-                                                     w.lb + kLbGaveUp, w.pert_idx, w.npert, w.st);
+                if ((r = radix_sort(c, sys->n, 1, &sk, &si, s, true)) != RV_OK) return r;
+                sel_member_write_k<<<M, 256, 0, s>>>(w.moff, sk, si, cap, C, j, w.lb + kLbGaveUp,
+                                                     w.pert_idx, w.npert, w.st);
                 count_launch(c);
             }
         }

@@ -204,7 +204,7 @@ rv_status upload_offsets(rv_ctx *c, int M, const int64_t *offsets, cudaStream_t 
 rv_status radix_sort(rv_ctx *c, int64_t n, int passes, uint64_t **keys, int **idx, cudaStream_t s,
                      bool member_pass = false, bool counted = false, const float4 *xyzm = nullptr,
                      float4 *pos = nullptr);
-rv_status exclusive_scan(rv_ctx *c, int *data, int64_t nmax, int *d_total, cudaStream_t s);   // *d_total: see scan_k
+rv_status exclusive_scan(rv_ctx *c, int *data, int64_t n, int *d_total, cudaStream_t s);   // *d_total: see scan_k
 int64_t sort_words(int64_t n_max);   // look-back words of a sort pass, for any n <= n_max
 
 // Layout of Workspace::lb (32-bit words): sort tickets [16], digit counts

@@ -96,3 +96,25 @@ def test_search_from_outside_is_no_slower_than_a_sort(centre, k):
         return min(t)
 
     assert best(k) <= 1.3 * best(6000)
+
+
+def test_members_without_perturbers():
+    """pert_k = 0 with several members: no perturbers, and no sort to select none."""
+    import torch
+    from paper_1507_01009_gb300 import rv
+    p32, m32 = hernquist32(9000, 44)
+    passes = {}
+    for mode, k in ((0, 0), (2, 0), (2, 5)):
+        S = rv.System(p32, np.zeros_like(p32), m32, chain_m=np.full(6, 0.01), chain_x=np.zeros((6, 3)) + 0.1,
+                      chain_v=np.zeros((6, 3)), pert_mode=mode, pert_k=k, member_offsets=[0, 2000, 2000, 9000],
+                      chains_per_member=2)
+        ctx = rv.Context(9000)
+        ctx.system_forces(S)
+        launched = ctx.launch_count()
+        a, pot = ctx.chain_perturber_forces(S, 0.0, S.chain_x)
+        ctx.sync_status()
+        passes[mode, k] = (launched, S.state[6:10].clone(), S.chain_a.clone(), a.clone())
+    assert passes[2, 0][0] == passes[0, 0][0]
+    for u, v in zip(passes[2, 0][1:], passes[0, 0][1:]):
+        assert torch.equal(u, v)
+    assert float(passes[2, 0][3].abs().max()) == 0.0 and float(passes[2, 5][3].abs().max()) > 0.0
