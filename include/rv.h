@@ -164,7 +164,12 @@ rv_status rv_tree_forces_rel(rv_ctx *ctx, float alpha, float eps_star, const flo
 /* rv_tree_forces after rv_build_tree_members: each star feels only its own
  * member's tree and the extra particles of its member; extra k belongs to
  * member extra_member[k] (device int32 [n_extra]; NULL = member 0) and walks
- * that member's tree. */
+ * that member's tree. A member's interactions are those of its stars alone;
+ * the order of its sums follows from the number of stars of the whole build
+ * (a group's walk is split into parts in builds of few stars), so its forces
+ * equal those of its stars alone bit for bit when both builds are walked in the
+ * same number of parts (always for members of 2^19 stars and more in groups of
+ * 64), and otherwise up to the rounding of compensated FP32 sums. */
 rv_status rv_tree_forces_members(rv_ctx *ctx, float theta, float eps_star, int32_t n_extra,
                                  const float *extra_xyzm, const float *extra_eps, const int32_t *extra_member,
                                  float *ax, float *ay, float *az, float *pot, float *extra_out, void *stream);
