@@ -50,10 +50,13 @@ constexpr int kMaxPert = 5000;
 // of 4096, 8192, 16384, 32768: 719, 614, 562, 643 / 1832, 1703, 1660, 1676;
 // unsplit 1286 / 1801.
 constexpr int kMaxParts = 16;
-// A single system of 2^17 to 2^19 stars takes twice as many: its full walks change
-// by -2 to +1 % (131072 stars 1105 -> 1086 us, 200001 1647 -> 1665), and the walks of
-// block time steps, in which few groups are active, by a quarter (sixteen
-// substeps of 200001 stars 12.4 -> 10.4 ms); an ensemble of that size loses 3 %.
+// A single system of 2^17 to 2^19 stars takes twice as many, for the walks of block
+// time steps: few groups are active in them, so that one item's time counts. A
+// masked walk gives the full walk's bits, so P cannot follow from the mask, and the
+// star count stands in for it. Full passes of 131072 / 200001 / 300000 / 400000 /
+// 520000 stars change by -2 / +0.9 / 0 / +0.1 / +0.2 % (1845, 2661, 3517, 4519 us of the
+// last four), sixteen substeps of 200001 / 300000 / 450000 stars 12.4 -> 10.5,
+// 19.3 -> 14.8, 22.2 -> 18.1 ms. A full pass of an ensemble of that size would lose 3 %.
 constexpr int kPartItems = 16384, kPartItemsMid = 2 * kPartItems;
 // Cells of more than 1 / kPartGrain of their member's stars are traversed by
 // every part (Part in walk.cu). Smaller subtrees balance better, larger ones
