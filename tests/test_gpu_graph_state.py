@@ -33,7 +33,7 @@ def _system(rvmod, sizes):
 
 
 @pytest.mark.parametrize("other", ["none", "build", "members", "search"])
-@pytest.mark.parametrize("sizes", [[3000], [9000], [2000, 3500, 5000]])
+@pytest.mark.parametrize("sizes", [[3000], [9000], [18000], [2000, 3500, 5000]])   # [18000]: a cluster searches
 def test_replay_after_other_builds(rvmod, sizes, other):
     import torch
     n, n_max = sum(sizes), 20000
