@@ -865,20 +865,26 @@ __device__ __forceinline__ void extra_terms(const WalkArgs &A, float xi, float y
     nadd(acc.ax, acc.cx, tx); nadd(acc.ay, acc.cy, ty); nadd(acc.az, acc.cz, tz); nadd(acc.ph, acc.cp, tp);
 }
 
-// A part of a walk is done: true in the warp that finishes the last of the P
-// parts (whose sums every part has then written), which also resets the counter.
-__device__ __forceinline__ bool last_part(int *arrive, int P) {
+// A part of a walk is done: nonzero in the warp that finishes the last of the P
+// parts (whose sums every part has then written), which also resets the counter; 1 if
+// every part's walk was whole, 2 if one was not (counted in the upper bits): then
+// the group's stars get no forces, as when an unsplit walk ends early.
+constexpr int kPartFailed = 1 << 16;
+__device__ __forceinline__ int last_part(int *arrive, int P, bool ok) {
     int last = 0;
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
         __threadfence();   // this part's sums before its arrival
-        last = atomicAdd(arrive, 1) == P - 1;
-        if (last) *arrive = 0;
+        const int old = atomicAdd(arrive, ok ? 1 : 1 + kPartFailed);
+        if ((old & (kPartFailed - 1)) == P - 1) {
+            last = ok && old < kPartFailed ? 1 : 2;
+            *arrive = 0;
+        }
         __threadfence();
     }
     last = __shfl_sync(0xffffffffu, last, 0);
     __syncwarp();   // the other parts' sums, acquired by lane 0, for every lane (a shuffle orders no memory)
-    return last != 0;
+    return last;
 }
 
 // A part's sums with their compensations (p: the part's slot of the star, `stride`
@@ -1062,7 +1068,7 @@ __global__ void RV_WALK_BOUNDS walk_tree_k(WalkArgs A) {
 #pragma unroll
             for (int h = 0; h < 2; h++)
                 if (lane + 32 * h < s) put_part(slot + (int64_t)2 * it.q * A.n + lane + 32 * h, A.n, tots[h]);
-            if (!last_part(A.garrive + it.group, P)) continue;
+            if (last_part(A.garrive + it.group, P, ok) != 1) continue;
 #pragma unroll
             for (int h = 0; h < 2; h++)
                 if (lane + 32 * h < s) tots[h] = add_parts(slot + lane + 32 * h, A.n, P);
